@@ -89,8 +89,9 @@ typedef struct {
     int32_t wave_levels;    /* AUTO: level cap of the top-down Evaluate before it hands over
                                to pointer jumping; 0 = tuned */
     int32_t host_loop;      /* 1 = drive the Replan loop from the host, one counter read per
-                               iteration; 0 = one CUDA-graph launch for the whole loop (a WHILE
-                               node repeats Improve / Evaluate on the device).  Profiling
+                               iteration; 0 = one launch for the whole loop (a cooperative
+                               kernel; with ASYNC, tile 1 .. 3 or other lane counts a CUDA
+                               graph whose WHILE node repeats Improve / Evaluate).  Profiling
                                always uses the host loop. */
     double dense_fraction;  /* changed vertices, as a fraction of |V|, above which the next
                                Improve sweeps every vertex instead of a list; 0 = tuned */
@@ -123,7 +124,10 @@ typedef struct {
  *            subtrees on its own and g is lowered by an atomic minimum, which
  *            no stale value can defeat because Improve never raises a
  *            cost-to-come (Sec. V policy improvement).  Same sums, bit for bit.
- *   AUTO  -- WAVE, handing over to JUMP when a wave exceeds its level cap. */
+ *   AUTO  -- without a goal, JUMP on graphs of up to 10^6 vertices (FP64 costs:
+ *            2 * 10^4, with the sums of the top 96 tree levels taken root to
+ *            leaf); else WAVE, handing over to JUMP when a wave exceeds its
+ *            level cap. */
 enum { PIRRT_EVAL_AUTO = 0, PIRRT_EVAL_WAVE = 1, PIRRT_EVAL_JUMP = 2, PIRRT_EVAL_ASYNC = 3 };
 
 /* Filled by pirrt_graph_exploit. */
@@ -140,7 +144,7 @@ typedef struct {
     int32_t wave_levels;    /* top-down Evaluate levels, summed over Evaluate calls */
     int32_t jump_evaluates; /* Evaluate calls done (or finished) by pointer jumping */
     float ms_exploit;       /* device time of the call, CUDA events on the graph's stream */
-    int32_t graph_launch;   /* 1 if the loop ran as one CUDA-graph launch */
+    int32_t graph_launch;   /* 1 if the whole loop ran as one launch (no host loop) */
     int64_t improve_entries; /* adjacency entries scanned by Improve alone (the relaxations of
                                a pull-only Improve); the same for every run of the same input */
     int64_t offers;         /* candidates formed by Evaluate for the next Improve (tile 0):
@@ -248,10 +252,8 @@ pirrt_status pirrt_graph_set_policy(pirrt_graph *g, const int32_t *parent, int64
  * minimum is kept and otherwise the lowest id wins.  Only vertices with a
  * neighbour whose g changed (or seeded by insertion) are re-examined.
  * Evaluate recomputes g(v) = g(p(v)) + c(p(v), v) in FP64 below the
- * switched vertices, by default top-down level by level (the wave of
- * PIRRT_EVAL_WAVE), handing over to pointer jumping when a wave passes its
- * level cap (PIRRT_EVAL_AUTO); see the Evaluate strategies above.  Blocks
- * until done; stats may be NULL.
+ * switched vertices, by pointer jumping or top-down level by level (see the
+ * Evaluate strategies above).  Blocks until done; stats may be NULL.
  * Errors: PIRRT_ERR_NOT_CONVERGED (max_iters reached; the state stays
  * consistent and exploit may be called again), PIRRT_ERR_BAD_TREE,
  * PIRRT_ERR_DEVICE_TIMEOUT, PIRRT_ERR_CUDA. */

@@ -108,6 +108,24 @@ __device__ __forceinline__ double widen(float w) {
 }
 __device__ __forceinline__ double widen(double w) { return w; }
 
+// Counters of one iteration of the persistent Replan loop (replan_loop.cuh).
+// Two sets take turns: CTA 0 clears the other one once every CTA is past its
+// last read of it, so no launch and no extra barrier resets them.
+constexpr unsigned kLoopIncomplete = 1u;  // a vertex was too deep to expand
+struct LoopCounters {
+    alignas(128) unsigned n_switched;
+    alignas(128) unsigned n_next;      // size of the list being built for the next Improve
+    alignas(128) unsigned n_dg;        // vertices whose g the wave changed
+    alignas(128) unsigned n_jump;      // vertices whose g pointer jumping changed
+    alignas(128) unsigned long long dj_bits;
+    alignas(128) unsigned wave_cnt[3];  // list sizes of grid steps t, t+1, t+2 (mod 3)
+    unsigned flags;                     // kLoopIncomplete
+};
+struct LoopState {  // CTA 0's totals of one exploit, read by the CTA that reports
+    unsigned long long switches;
+    unsigned iter, converged, wave_levels, dense_sweeps, jump_rounds, jump_evals;
+};
+
 // Device counters of one graph.  The host copies the block back once per
 // Replan iteration.
 // Counters that every CTA of a kernel adds to sit on 128-byte lines of
@@ -158,6 +176,11 @@ struct DevCounters {
     unsigned last_switched, last_dg, last_levels, last_next, last_dense, last_rounds, last_jumped;
     // whole-exploit totals
     unsigned cum_wave_levels, cum_dense, cum_jump_rounds, cum_jump_evals;
+    // persistent loop
+    alignas(128) unsigned long long loop_bar[32];  // its barrier's two words, a line each
+    LoopCounters loop[2];
+    LoopState loop_state;
+    unsigned loop_par;            // which counter set the next iteration uses
     // Level trace, kept while profiling is on (lvl_trace = 1) and left alone
     // by a reset of the graph: the top-down Evaluate's levels by size bucket,
     // the vertices they held and CTA 0's SM cycles over them (each level's

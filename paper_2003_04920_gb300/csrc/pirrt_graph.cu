@@ -2,11 +2,11 @@
 //
 // All graph state (CSR, g, parents, work lists) stays resident on the
 // device.  A Replan (Alg. 2: Improve, then Evaluate, until no parent
-// switches) runs as one CUDA-graph launch whose WHILE node repeats the loop
-// body on the device -- Improve, then Evaluate, which ends the iteration by
-// testing convergence and setting the loop condition -- so the host waits
-// once per exploit.  With profiling enabled the same kernels run from a host
-// loop that reads the counter block after every iteration.
+// switches) runs as one cooperative launch (replan_loop.cuh), so the host waits
+// once per exploit.  Non-default kernel choices run as one CUDA-graph launch
+// whose WHILE node repeats an iteration's kernels, and with profiling enabled
+// those kernels run from a host loop that reads the counter block after every
+// iteration.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,6 +26,7 @@
 #include "improve_screen.cuh"
 #include "improve_tma.cuh"
 #include "replan_iteration.cuh"
+#include "replan_loop.cuh"
 #include "pirrt.h"
 
 using namespace pirrt;
@@ -115,6 +116,10 @@ struct pirrt_graph {
     void *stage = nullptr;            // device staging for host-side inputs
     size_t stage_bytes = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+    WaveItem *items[2] = {nullptr, nullptr};  // persistent loop: grid-step lists
+    JumpRec *rec[2] = {nullptr, nullptr};     // ... pointer-jumping records
+    LoopResult *loop_res = nullptr;           // ... what an exploit reports (pinned)
+    int loop_occ = 0;                         // ... CTAs per SM (<= 2)
     int eval_blocks = 0;
     int wave_blocks = 0;                  // grid of the wave for the current exploit
     int wave_occ = 0;                     // CTAs per SM the wave can keep resident (<= 2)
@@ -460,7 +465,7 @@ pirrt_status launch_evaluate(pirrt_graph *G, cudaStream_t st, size_t off) {
 // when fused_improve is set.
 template <typename CT>
 pirrt_status launch_wave(pirrt_graph *G, cudaStream_t st, cudaGraphConditionalHandle cond,
-                         int use_cond, bool fused_improve = false, bool fuse_dense = false) {
+                         int use_cond, bool fused_improve = false) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(G->wave_blocks);
     cfg.blockDim = dim3(kWaveThreads);
@@ -474,25 +479,17 @@ pirrt_status launch_wave(pirrt_graph *G, cudaStream_t st, cudaGraphConditionalHa
     const ImproveArgs<CT> *ip = fused_improve ? dev_arg<ImproveArgs<CT>>(G, kArgImprove) : nullptr;
     CK(cudaLaunchKernelEx(&cfg, wave_evaluate_kernel<CT>, dev_arg<WaveArgs<CT>>(G, kArgWave),
                           dev_arg<EvaluateArgs<CT>>(G, kArgEvalFallback),
-                          dev_arg<MarkArgs<CT>>(G, kArgMarkFallback), ip, cond, use_cond,
-                          fuse_dense ? 1 : 0));
+                          dev_arg<MarkArgs<CT>>(G, kArgMarkFallback), ip, cond, use_cond));
     return PIRRT_OK;
 }
 
-// A captured iteration with offers whose dense sweeps run inside the wave's
-// launch too (FP32 costs, the default 4 lanes): one launch per iteration.
-bool fuses_dense(int cost_dtype, int tile, int gs) {
-    return cost_dtype == PIRRT_COST_F32 && tile == 0 && (gs == 0 || gs == 4);
-}
-
 // Kernel launches of one Replan iteration (host loop; a captured wave
-// iteration with offers runs the offer Improve inside the wave's launch, and
-// with FP32 costs the dense sweep as well).
-int iteration_launches(int tile, bool jump, bool async, bool graph, bool fused_dense = false) {
+// iteration with offers runs the offer Improve inside the wave's launch).
+int iteration_launches(int tile, bool jump, bool async, bool graph) {
     const int improve = tile == 0 ? 2 : 1;
     if (jump) return improve + 3;
     if (async) return improve + 5;
-    if (graph && tile == 0) return fused_dense ? 1 : 2;
+    if (graph && tile == 0) return 2;
     return improve + 1;
 }
 
@@ -532,9 +529,7 @@ pirrt_status launch_iteration(pirrt_graph *G, cudaStream_t st, int gs, int tile,
     pirrt_status rc;
     if (!jump && !async && tile == 0) {
         // the dense-sweep kernel, then Improve from offers and the wave in one
-        // launch; with FP32 costs that launch also runs the dense sweeps
-        if (fuses_dense(G->cfg.cost_dtype, tile, gs))
-            return launch_wave<CT>(G, st, cond, use_cond, true, true);
+        // launch
         if ((rc = launch_improve<CT>(G, st, gs, tile, false))) return rc;
         return launch_wave<CT>(G, st, cond, use_cond, true);
     }
@@ -741,6 +736,107 @@ pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const i
     return PIRRT_OK;
 }
 
+// Goal-free graphs up to this size evaluate by pointer jumping in AUTO: its cost
+// grows with the graph (20 us an iteration at 2*10^5 vertices, 50 at 10^6) where
+// a wave's is the depth of the change (40 to 130 us on the 2-D and 6-D roadmaps).
+// With a goal the wave prunes and pointer jumping does not.
+// FP64 costs, whose sums round, first take kTopRounds rounds that add from the
+// root down like the wave (96 tree levels, the depth of 2-D roadmaps of about
+// this size), so that only deeper vertices get reassociated sums.
+constexpr int64_t kJumpVertices = 1000000, kJumpVerticesF64 = 20000;
+constexpr int kTopRounds = 8;
+
+// The default exploit: the whole Replan loop as one cooperative launch
+// (replan_loop.cuh).  One host wait, no read-back copy: the kernel leaves its
+// report in page-locked host memory.
+template <typename CT>
+pirrt_status exploit_loop(pirrt_graph *G, const pirrt_exploit_opts &o, bool jump, bool adaptive,
+                          int top_rounds, int64_t max_iters, unsigned dense_limit, unsigned max_levels,
+                          pirrt_exploit_stats *st) {
+    LoopArgs<CT> a{};
+    a.rows = G->rows;
+    a.adj = static_cast<const Entry<CT> *>(G->adj[G->cur]);
+    a.g = G->g;
+    a.g32 = G->g32;
+    a.p = G->p;
+    a.pc = static_cast<CT *>(G->pc);
+    a.cand = G->cand;
+    a.stamp = G->stamp;
+    a.wstamp = G->wstamp;
+    a.dg = G->dg;
+    for (int k = 0; k < 2; ++k) {
+        a.list[k] = G->list[k];
+        a.items[k] = G->items[k];
+        a.rec[k] = G->rec[k];
+    }
+    a.ctr = G->ctr;
+    a.res = G->loop_res;
+    a.h = G->goal >= 0 ? G->h : nullptr;
+    a.goal_g = G->goal >= 0 ? G->g + G->goal : nullptr;
+    a.eps = o.eps;
+    a.n = G->n;
+    a.list_cap = G->cap_n;
+    a.root = G->cfg.root;
+    a.jump = jump ? 1 : 0;
+    a.top_rounds = top_rounds;
+    a.hops = G->n <= 50000 ? 7 : (G->n <= 1000000 ? 3 : 2);
+    a.max_iters = (unsigned)std::min<int64_t>(max_iters, 0xffffffffll);
+    a.dense_limit = dense_limit;
+    a.max_levels = max_levels;
+    a.tail_max = o.wave_tail > 0 ? (unsigned)o.wave_tail : 0u;
+    a.local_levels = o.wave_local < 0 ? 0u : (o.wave_local > 0 ? (unsigned)o.wave_local : 32u);
+    a.local_max = o.wave_local_max > 0 ? (unsigned)o.wave_local_max : 32u;
+    a.local_step = o.wave_local_step > 0 ? (unsigned)o.wave_local_step : 512u;
+    const int occ = o.wave_ctas > 0 ? std::min(o.wave_ctas, G->loop_occ) : G->loop_occ;
+    int blocks = G->num_sms * occ;
+    blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(8, (G->n + 127) / 128));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kLoopThreads);
+    cfg.dynamicSmemBytes = sizeof(LoopShared<CT>);
+    cfg.stream = G->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CK(cudaEventRecord(G->ev0, G->stream));
+    CK(cudaLaunchKernelEx(&cfg, replan_loop_kernel<CT>, a));
+    CK(cudaEventRecord(G->ev1, G->stream));
+    CK(cudaStreamSynchronize(G->stream));
+    G->prof.launches += 1;
+    const LoopResult r = *G->loop_res;
+    float ms = 0.f;
+    CK(cudaEventElapsedTime(&ms, G->ev0, G->ev1));
+    G->ctr_host->wave_epoch = r.wave_epoch;
+    if (adaptive) {
+        const bool saw_deep = r.jump_evals > 0;
+        if (saw_deep || !jump || (G->exploits % 8) == 1) G->deep_hint = saw_deep ? 1 : 0;
+    }
+    pirrt_exploit_stats s{};
+    s.iterations = (int32_t)r.iter;
+    s.converged = r.converged ? 1 : 0;
+    s.relaxations = (int64_t)(r.relax + r.offers);
+    s.improve_entries = (int64_t)r.relax;
+    s.offers = (int64_t)r.offers;
+    s.improved = (int64_t)r.improved;
+    s.evaluated = (int64_t)r.evaluated;
+    s.switches = (int64_t)r.switches;
+    s.jump_rounds = (int32_t)r.jump_rounds;
+    s.dense_sweeps = (int32_t)r.dense_sweeps;
+    s.wave_levels = (int32_t)r.wave_levels;
+    s.jump_evaluates = (int32_t)r.jump_evals;
+    s.ms_exploit = ms;
+    s.graph_launch = 1;
+    if (st) *st = s;
+    if (r.status & kStatusTimeout) G->recover = 1;
+    if (const pirrt_status rc = status_from_bits(G, r.status)) return rc;
+    if (!r.converged)
+        return fail(G, PIRRT_ERR_NOT_CONVERGED, "exploit: %lld Improve rounds without convergence",
+                    (long long)max_iters);
+    return PIRRT_OK;
+}
+
 template <typename CT>
 pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_exploit_stats *st) {
     pirrt_exploit_opts o{};
@@ -759,6 +855,9 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
         // (every vertex), so that the next Improve starts from a consistent
         // state and sweeps every vertex
         CK(cudaMemsetAsync(&G->ctr->status, 0, sizeof(unsigned), G->stream));
+        CK(cudaMemsetAsync(&G->ctr->wave_ticket, 0, sizeof(unsigned), G->stream));
+        CK(cudaMemsetAsync(G->ctr->loop, 0, sizeof(G->ctr->loop), G->stream));
+        CK(cudaMemsetAsync(G->ctr->loop_bar, 0, sizeof(G->ctr->loop_bar), G->stream));
         const pirrt_status rr = reevaluate_impl<CT>(G);
         if (rr) return rr;
         G->recover = 0;
@@ -797,6 +896,9 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
     // jumping; probe with a wave again every eighth exploit
     bool jump = mode == PIRRT_EVAL_JUMP ||
                 (mode == PIRRT_EVAL_AUTO && G->deep_hint && (G->exploits % 8) != 0);
+    const bool small = mode == PIRRT_EVAL_AUTO && G->goal < 0 &&
+                       G->n <= (sizeof(CT) == 8 ? kJumpVerticesF64 : kJumpVertices);
+    if (small) jump = true;
     G->exploits += 1;
     // one CTA walks levels of at most this many vertices (~34 CSR entries each
     // on the 6-D roadmaps, a few passes of the CTA's threads)
@@ -808,6 +910,10 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
         o.wave_local < 0 ? 0u : (o.wave_local > 0 ? (unsigned)o.wave_local : 32u);
     const unsigned local_max = o.wave_local_max > 0 ? (unsigned)o.wave_local_max : 128u;
     const unsigned local_step = o.wave_local_step > 0 ? (unsigned)o.wave_local_step : 4096u;
+    if (G->profiling != 1 && o.host_loop == 0 && tile == 0 && !async &&
+        (sizeof(CT) == 8 || gs == 0 || gs == 4))
+        return exploit_loop<CT>(G, o, jump, mode == PIRRT_EVAL_AUTO && !small,
+                                small ? kTopRounds : 0, max_iters, dense_limit, max_levels, st);
     pirrt_status rc = write_args<CT>(G, dense_limit, max_levels, tile == 0 ? 1 : 0, tail_max,
                                      local_levels, local_max, local_step);
     if (rc) return rc;
@@ -947,8 +1053,7 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
         if (saw_deep || !jump || (G->exploits % 8) == 1) G->deep_hint = saw_deep ? 1 : 0;
     }
     if (graph_ran)
-        P.launches += (int64_t)h.iter * iteration_launches(tile, jump, async, true,
-                                                            fuses_dense(G->cfg.cost_dtype, tile, gs));
+        P.launches += (int64_t)h.iter * iteration_launches(tile, jump, async, true);
     s.iterations = (int32_t)h.iter;
     s.converged = h.converged ? 1 : 0;
     s.relaxations = (int64_t)(h.relax + h.offers);
@@ -1051,11 +1156,13 @@ void free_all(pirrt_graph *G) {
     void *bufs[] = {G->dargs, G->pexport, G->rows, G->ralloc, G->touched, G->roff, G->adj[0], G->adj[1], G->g, G->g32, G->p, G->pc,
                     G->deg, G->tile_sums, G->stamp, G->list[0], G->list[1], G->switched,
                     G->dg, G->anc[0], G->anc[1], G->acc[0], G->acc[1], G->wx[0], G->wx[1], G->done, G->wl[0],
-                    G->wl[1], G->wstamp, G->swstamp, G->cand, G->aq, G->aring, G->ctr, G->stage, G->h};
+                    G->wl[1], G->wstamp, G->swstamp, G->cand, G->aq, G->aring, G->ctr, G->stage, G->h,
+                    G->items[0], G->items[1], G->rec[0], G->rec[1]};
     for (void *q : bufs)
         if (q) cudaFree(q);
     if (G->ctr_host) cudaFreeHost(G->ctr_host);
     if (G->hx) cudaFreeHost(G->hx);
+    if (G->loop_res) cudaFreeHost(G->loop_res);
     if (G->ev0) cudaEventDestroy(G->ev0);
     if (G->ev1) cudaEventDestroy(G->ev1);
     for (cudaEvent_t e : G->pev)
@@ -1256,6 +1363,10 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     ALLOC(G->ctr, sizeof(DevCounters));
     ALLOC(G->dargs, kArgBytes);
     ALLOC(G->pexport, sizeof(int32_t) * nv);
+    for (int k = 0; k < 2; ++k) {
+        ALLOC(G->items[k], sizeof(WaveItem) * nv);
+        ALLOC(G->rec[k], sizeof(JumpRec) * nv);
+    }
 #undef ALLOC
     if (cudaMallocHost((void **)&G->hargs, kArgBytes) != cudaSuccess) return bail(PIRRT_ERR_OOM);
     if (cudaStreamCreateWithFlags(&G->copy, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1267,6 +1378,8 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     if (cudaMallocHost((void **)&G->hx, 2 * sizeof(int64_t)) != cudaSuccess)
         return bail(PIRRT_ERR_OOM);
     if (cudaMallocHost((void **)&G->ctr_host, sizeof(DevCounters)) != cudaSuccess)
+        return bail(PIRRT_ERR_OOM);
+    if (cudaMallocHost((void **)&G->loop_res, sizeof(LoopResult)) != cudaSuccess)
         return bail(PIRRT_ERR_OOM);
     if (cudaEventCreate(&G->ev0) != cudaSuccess || cudaEventCreate(&G->ev1) != cudaSuccess)
         return bail(PIRRT_ERR_CUDA);
@@ -1296,6 +1409,20 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     if (wocc < 1) return bail(PIRRT_ERR_CUDA);
     G->wave_occ = std::min(wocc, 2);
     G->wave_blocks = G->num_sms * G->wave_occ;
+    int locc = 0, locc64 = 0;
+    if (cudaFuncSetAttribute(replan_loop_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(LoopShared<float>)) != cudaSuccess ||
+        cudaFuncSetAttribute(replan_loop_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(LoopShared<double>)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&locc, replan_loop_kernel<float>, kLoopThreads,
+                                                      sizeof(LoopShared<float>)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&locc64, replan_loop_kernel<double>,
+                                                      kLoopThreads, sizeof(LoopShared<double>)) !=
+            cudaSuccess)
+        return bail(PIRRT_ERR_CUDA);
+    locc = std::min(locc, locc64);
+    if (locc < 1) return bail(PIRRT_ERR_CUDA);
+    G->loop_occ = std::min(locc, 2);
     int aocc = 0, aocc64 = 0;
     if (cudaFuncSetAttribute(async_evaluate_kernel<float>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAsyncSmem) !=
