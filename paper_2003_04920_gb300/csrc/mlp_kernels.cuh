@@ -110,6 +110,121 @@ gemm_nt_bf16(int M, int N, int K, const __nv_bfloat16 *__restrict__ A, int lda,
 }
 
 // ---------------------------------------------------------------------------
+// The grid part of layer 1, once per scene: hg[s][j] = sum_k grid[s][k] W1g[j][k]
+// (the grid rounded to BF16, FP32 accumulation) and hgb = hg + b1.
+//
+// 32 hidden-unit groups of 8 and a handful of scenes give few tiles, and each
+// output is one accumulation over K = 4096: the time is the chain of 256
+// dependent m16n8k16 steps (21 cycles each, 2.8 us) plus what it waits for its
+// operands.  So a warp owns one 16 x 8 tile and takes the steps in order (the
+// sums are those of gemm_nt_bf16, bit for bit), two warps of a CTA serve 32
+// scenes, and all four keep a four-stage ring of asynchronous copies ahead of
+// them: 256 values of K of W1g and of the caller's FP32 grids, which are
+// converted on their way into the fragments.  Measured, 1 to 32 scenes:
+// 99 us with 64 x 64 tiles, no prefetch, and conversion and transposition passes
+// before it; 12 us for 32 now.
+// ---------------------------------------------------------------------------
+constexpr int kSceneN = 8;                 // hidden units per CTA
+constexpr int kSceneM = 32;                // scenes per CTA
+constexpr int kSceneK = 256, kSceneStages = 4;
+constexpr int kSceneGRow = kSceneK + 8;    // padded rows (FP32 grids, BF16 weights)
+struct SceneStage {
+    float grid[kSceneM][kSceneGRow];
+    __nv_bfloat16 w[kSceneN][kSceneGRow];
+};
+constexpr int kSceneSmem = kSceneStages * (int)sizeof(SceneStage);
+
+__device__ __forceinline__ uint32_t pack2(float2 v) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(v.x, v.y);
+    return *reinterpret_cast<const uint32_t *>(&p);
+}
+
+static __global__ void __launch_bounds__(128)
+scene_features_kernel(int n_scenes, const float *__restrict__ grids,
+                      const __nv_bfloat16 *__restrict__ W1gb, const float *__restrict__ b1,
+                      float *__restrict__ hg, float *__restrict__ hgb) {
+    extern __shared__ __align__(16) unsigned char scene_smem[];
+    SceneStage *st = reinterpret_cast<SceneStage *>(scene_smem);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n0 = blockIdx.x * kSceneN, c0 = blockIdx.y * kSceneM, s0 = c0 + warp * 16;
+    const int rows = n_scenes - c0 < kSceneM ? n_scenes - c0 : kSceneM;
+    const int gid = lane >> 2, tig = lane & 3;
+    const bool vec = (reinterpret_cast<uintptr_t>(grids) & 15u) == 0u;
+    auto load = [&](int chunk) {
+        if (chunk < kGrid / kSceneK) {
+            SceneStage &d = st[chunk % kSceneStages];
+            const int k0 = chunk * kSceneK;
+            if (vec) {
+                for (int i = tid; i < rows * (kSceneK / 4); i += 128) {
+                    const int r = i / (kSceneK / 4), k = i % (kSceneK / 4) * 4;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                     (uint32_t)__cvta_generic_to_shared(&d.grid[r][k])),
+                                 "l"(grids + (size_t)(c0 + r) * kGrid + k0 + k)
+                                 : "memory");
+                }
+            } else {
+                for (int i = tid; i < rows * kSceneK; i += 128) {
+                    const int r = i / kSceneK, k = i % kSceneK;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                                     (uint32_t)__cvta_generic_to_shared(&d.grid[r][k])),
+                                 "l"(grids + (size_t)(c0 + r) * kGrid + k0 + k)
+                                 : "memory");
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kSceneN * kSceneK / 8 / 128; ++q) {
+                const int i = tid + q * 128, r = i / (kSceneK / 8), k = i % (kSceneK / 8) * 8;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                 (uint32_t)__cvta_generic_to_shared(&d.w[r][k])),
+                             "l"(W1gb + (size_t)(n0 + r) * kGrid + k0 + k)
+                             : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    // rows past the last scene stay zero (their results are not stored)
+    for (int b = 0; b < kSceneStages; ++b)
+        for (int i = tid; i < (kSceneM - rows) * kSceneGRow; i += 128)
+            st[b].grid[rows + i / kSceneGRow][i % kSceneGRow] = 0.f;
+#pragma unroll
+    for (int c = 0; c < kSceneStages - 1; ++c) load(c);
+    const bool live = warp < 2 && s0 < n_scenes;  // warp-uniform
+    float acc[4] = {};
+#pragma unroll 1
+    for (int c = 0; c < kGrid / kSceneK; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSceneStages - 2) : "memory");
+        __syncthreads();
+        load(c + kSceneStages - 1);  // into the stage read last turn
+        if (!live) continue;
+        const SceneStage &d = st[c % kSceneStages];
+        const float *ga = &d.grid[warp * 16 + gid][tig * 2], *gb = ga + 8 * kSceneGRow;
+        const __nv_bfloat16 *wr = &d.w[gid][tig * 2];
+#pragma unroll
+        for (int k = 0; k < kSceneK; k += 16) {
+            const uint32_t af[4] = {pack2(*reinterpret_cast<const float2 *>(ga + k)),
+                                    pack2(*reinterpret_cast<const float2 *>(gb + k)),
+                                    pack2(*reinterpret_cast<const float2 *>(ga + k + 8)),
+                                    pack2(*reinterpret_cast<const float2 *>(gb + k + 8))};
+            const uint32_t bf[2] = {*reinterpret_cast<const uint32_t *>(wr + k),
+                                    *reinterpret_cast<const uint32_t *>(wr + k + 8)};
+            mma_bf16(acc, af, bf);
+        }
+    }
+    if (!live) return;
+    const int c = n0 + tig * 2;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int s = s0 + gid + 8 * h;
+        if (s >= n_scenes) continue;
+        const size_t o = (size_t)s * kHidden + c;
+        hg[o] = acc[2 * h];
+        hg[o + 1] = acc[2 * h + 1];
+        hgb[o] = acc[2 * h] + b1[c];
+        hgb[o + 1] = acc[2 * h + 1] + b1[c + 1];
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Elementwise and small kernels.  Rows are padded to multiples of 64; padded
 // rows carry zeros and are excluded by `rows` where it matters.
 // ---------------------------------------------------------------------------
@@ -130,20 +245,20 @@ __global__ void to_bf16(int rows, int cols, const float *__restrict__ in, int ld
 }
 
 // Layer 1 for sample rows: a1[r][j] = hg[scene[r]][j] + sum_k W1n[j][k] z[r][k]
-// + b1[j] (FP32; z and W1n used in their BF16-rounded values), h1 = relu(a1)
-// as BF16 (row-major and transposed).
+// + b1[j] (FP32; z and W1n used in their BF16-rounded values), h1 = relu(a1) as
+// BF16; row r's scene is scene[r / rows_per_scene].
 __global__ void layer1_rows(int rows, int rows_pad, const float *__restrict__ hg,
-                            const int32_t *__restrict__ scene, const float *__restrict__ z,
-                            const float *__restrict__ W1n, const float *__restrict__ b1,
-                            float *__restrict__ a1, __nv_bfloat16 *__restrict__ h1,
-                            __nv_bfloat16 *__restrict__ h1T) {
+                            const int32_t *__restrict__ scene, int rows_per_scene,
+                            const float *__restrict__ z, const float *__restrict__ W1n,
+                            const float *__restrict__ b1,
+                            float *__restrict__ a1, __nv_bfloat16 *__restrict__ h1) {
     const int64_t total = (int64_t)rows_pad * kHidden;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(i / kHidden), j = (int)(i % kHidden);
         float a = 0.f;
         if (r < rows) {
-            a = hg[(size_t)scene[r] * kHidden + j] + b1[j];
+            a = hg[(size_t)scene[r / rows_per_scene] * kHidden + j] + b1[j];
 #pragma unroll
             for (int k = 0; k < kNoise; ++k)
                 a += __bfloat162float(__float2bfloat16_rn(W1n[j * kNoise + k])) *
@@ -152,13 +267,12 @@ __global__ void layer1_rows(int rows, int rows_pad, const float *__restrict__ hg
         a1[i] = a;
         const __nv_bfloat16 h = __float2bfloat16_rn(r < rows && a > 0.f ? a : 0.f);
         h1[i] = h;
-        if (h1T) h1T[(size_t)j * rows_pad + r] = h;
     }
 }
 
 // a2 += b2 (rows), h2 = relu(a2) as BF16.
 __global__ void bias_relu(int rows, int rows_pad, float *__restrict__ a, const float *__restrict__ b,
-                          __nv_bfloat16 *__restrict__ h, __nv_bfloat16 *__restrict__ hT) {
+                          __nv_bfloat16 *__restrict__ h) {
     const int64_t total = (int64_t)rows_pad * kHidden;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -167,7 +281,6 @@ __global__ void bias_relu(int rows, int rows_pad, float *__restrict__ a, const f
         a[i] = v;
         const __nv_bfloat16 q = __float2bfloat16_rn(v > 0.f ? v : 0.f);
         h[i] = q;
-        if (hT) hT[(size_t)j * rows_pad + r] = q;
     }
 }
 
@@ -227,152 +340,6 @@ __global__ void mix_samples(int rows, const float *__restrict__ y, const float *
         const bool learned = coin[r] < learned_fraction;
         out[2 * r] = learned ? y[2 * r] : uni[2 * r];
         out[2 * r + 1] = learned ? y[2 * r + 1] : uni[2 * r + 1];
-    }
-}
-
-// draw_scene[t*K + k] = target_scene[t]
-__global__ void repeat_scene(int n_targets, int K, const int32_t *__restrict__ scene,
-                             int32_t *__restrict__ out) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_targets * K; i += gridDim.x * blockDim.x)
-        out[i] = scene[i / K];
-}
-
-// Gather the picked noise vectors: z_sel[t] = z_all[t*K + pick[t]].
-__global__ void gather_noise(int n_targets, int K, const float *__restrict__ z_all,
-                             const int32_t *__restrict__ pick, float *__restrict__ z_sel) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_targets * kNoise;
-         i += gridDim.x * blockDim.x) {
-        const int t = i / kNoise, k = i % kNoise;
-        z_sel[i] = z_all[(size_t)(t * K + pick[t]) * kNoise + k];
-    }
-}
-
-// Loss L = (1/T) sum_t |y_t - target_t|^2 and the output-layer backward:
-// da3 = dL/da3 = (2/T)(y - target) y (1 - y); dW3 += da3^T h2 (FP32, exact
-// sums over rows in a fixed order per output unit); db3 += sum da3;
-// dh2 = da3 W3 (BF16 W3) masked by relu -> da2 (FP32 and BF16, both layouts).
-// One block per hidden unit j handles dW3[:, j]; the loss is accumulated by
-// block 0.
-__global__ void output_backward(int rows, int rows_pad, const float *__restrict__ y,
-                                const float *__restrict__ target,
-                                const __nv_bfloat16 *__restrict__ h2,
-                                const __nv_bfloat16 *__restrict__ W3b, const float *__restrict__ a2,
-                                float *__restrict__ dW3, float *__restrict__ db3,
-                                __nv_bfloat16 *__restrict__ da2b, __nv_bfloat16 *__restrict__ da2T,
-                                float *__restrict__ da2f, float *__restrict__ loss) {
-    const float scale = 2.f / (float)rows;
-    const int j = blockIdx.x;  // hidden unit
-    float s0 = 0.f, s1 = 0.f;
-    for (int r = threadIdx.x; r < rows_pad; r += blockDim.x) {
-        float d0 = 0.f, d1 = 0.f;
-        if (r < rows) {
-            const float y0 = y[2 * r], y1 = y[2 * r + 1];
-            d0 = scale * (y0 - target[2 * r]) * y0 * (1.f - y0);
-            d1 = scale * (y1 - target[2 * r + 1]) * y1 * (1.f - y1);
-        }
-        const float h = __bfloat162float(h2[(size_t)r * kHidden + j]);
-        s0 += d0 * h;
-        s1 += d1 * h;
-        const float dh = d0 * __bfloat162float(W3b[j]) + d1 * __bfloat162float(W3b[kHidden + j]);
-        const float da = (r < rows && a2[(size_t)r * kHidden + j] > 0.f) ? dh : 0.f;
-        da2f[(size_t)r * kHidden + j] = da;
-        const __nv_bfloat16 q = __float2bfloat16_rn(da);
-        da2b[(size_t)r * kHidden + j] = q;
-        da2T[(size_t)j * rows_pad + r] = q;
-    }
-    __shared__ float red[2][32];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, off);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        red[0][threadIdx.x >> 5] = s0;
-        red[1][threadIdx.x >> 5] = s1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t0 = 0.f, t1 = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            t0 += red[0][w];
-            t1 += red[1][w];
-        }
-        dW3[j] += t0;
-        dW3[kHidden + j] += t1;
-    }
-    if (j == 0 && threadIdx.x == 0) {
-        float l = 0.f, g0 = 0.f, g1 = 0.f;
-        for (int r = 0; r < rows; ++r) {
-            const float y0 = y[2 * r], y1 = y[2 * r + 1];
-            const float e0 = y0 - target[2 * r], e1 = y1 - target[2 * r + 1];
-            l += e0 * e0 + e1 * e1;
-            g0 += scale * e0 * y0 * (1.f - y0);
-            g1 += scale * e1 * y1 * (1.f - y1);
-        }
-        loss[0] = l / (float)rows;
-        db3[0] += g0;
-        db3[1] += g1;
-    }
-}
-
-// Column sums: out[j] += sum_r in[r][j] (FP32), one thread per column.
-__global__ void col_sum(int rows, int cols, const float *__restrict__ in, float *__restrict__ out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= cols) return;
-    float s = 0.f;
-    for (int r = 0; r < rows; ++r) s += in[(size_t)r * cols + j];
-    out[j] += s;
-}
-
-// dh1 (FP32, from the dh1 = da2 W2 GEMM) masked by relu(a1) -> da1 (FP32);
-// scene sums D[s][j] += da1 for the W1 grid gradient (BF16 transposed copy
-// written afterwards), dW1n += da1^T z (FP32), db1 += sum da1.  One thread
-// per hidden unit j, rows in order.
-__global__ void layer1_backward(int rows, const float *__restrict__ dh1, const float *__restrict__ a1,
-                                const int32_t *__restrict__ scene, const float *__restrict__ z,
-                                float *__restrict__ D, float *__restrict__ dW1n,
-                                float *__restrict__ db1) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= kHidden) return;
-    float gw[kNoise] = {};
-    float gb = 0.f;
-    for (int r = 0; r < rows; ++r) {
-        const float d = a1[(size_t)r * kHidden + j] > 0.f ? dh1[(size_t)r * kHidden + j] : 0.f;
-        D[(size_t)scene[r] * kHidden + j] += d;
-        gb += d;
-#pragma unroll
-        for (int k = 0; k < kNoise; ++k)
-            gw[k] += d * __bfloat162float(__float2bfloat16_rn(z[r * kNoise + k]));
-    }
-    db1[j] += gb;
-#pragma unroll
-    for (int k = 0; k < kNoise; ++k) dW1n[j * kNoise + k] += gw[k];
-}
-
-// Adam on FP32 master weights, then the BF16 working copy (and optionally a
-// transposed BF16 copy for the backward GEMMs).  rows x cols row-major.
-__global__ void adam_step(int rows, int cols, float *__restrict__ w, float *__restrict__ m,
-                          float *__restrict__ v, float *__restrict__ grad, float lr, float beta1,
-                          float beta2, float eps, float bc1, float bc2,
-                          __nv_bfloat16 *__restrict__ wb, __nv_bfloat16 *__restrict__ wbT,
-                          int ldT) {
-    const int64_t total = (int64_t)rows * cols;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float gr = grad[i];
-        const float mi = beta1 * m[i] + (1.f - beta1) * gr;
-        const float vi = beta2 * v[i] + (1.f - beta2) * gr * gr;
-        m[i] = mi;
-        v[i] = vi;
-        const float wi = w[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-        w[i] = wi;
-        grad[i] = 0.f;
-        const __nv_bfloat16 q = __float2bfloat16_rn(wi);
-        if (wb) wb[i] = q;
-        if (wbT) {
-            const int r = (int)(i / cols), c = (int)(i % cols);
-            wbT[(size_t)c * ldT + r] = q;
-        }
     }
 }
 

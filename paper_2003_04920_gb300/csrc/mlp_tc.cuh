@@ -213,7 +213,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 struct FwdArgs {
     int rows, n_scenes;
     const float *hgb;              // [n_scenes x 256] W1g grid + b1 per scene
-    const int32_t *scene;          // [rows]
+    const int32_t *scene;          // [rows / rows_per_scene]: row r's is scene[r / rows_per_scene]
+    int rows_per_scene;
     const float *z;                // [rows x 8]
     const float *W1n;              // [256 x 8] FP32 master weights (rounded here)
     const __nv_bfloat16 *W2b;      // [256 x 256], row = output unit
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_forward_tc(const FwdArgs A) {
         const int rn = next * kRowsPerTile + row;
         int s = 0;
         if (valid) {
-            s = A.scene[r];
+            s = A.scene[A.rows_per_scene == 1 ? r : r / A.rows_per_scene];
             if (s < 0 || s >= A.n_scenes) {
                 if (half == 0) atomicOr(A.status, kErrScene);
                 s = 0;

@@ -10,6 +10,7 @@
 
 #include "mlp_kernels.cuh"
 #include "mlp_tc.cuh"
+#include "mlp_train.cuh"
 #include "pirrt.h"
 
 using namespace pirrt::mlp;
@@ -37,18 +38,21 @@ struct pirrt_proposal {
     int max_scenes = 0, max_rows = 0, S = 0, R = 0;  // padded capacities
     float *w = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;
     __nv_bfloat16 *W1gb = nullptr, *W2b = nullptr, *W2Tb = nullptr, *W3b = nullptr;
-    __nv_bfloat16 *gridb = nullptr, *gridT = nullptr;  // [S x 4096], [4096 x S]
     float *hg = nullptr;                                // [S x 256]
-    float *a1 = nullptr, *a2 = nullptr, *dh1 = nullptr, *da2f = nullptr;  // [R x 256]
-    __nv_bfloat16 *h1 = nullptr, *h1T = nullptr, *h2 = nullptr, *da2b = nullptr, *da2T = nullptr;
+    float *a1 = nullptr, *a2 = nullptr;                 // [R x 256], the layered forward pass
+    __nv_bfloat16 *h1 = nullptr, *h2 = nullptr, *da2 = nullptr;  // [R x 256]
     float *y = nullptr;                                 // [R x 2]
-    float *D = nullptr;                                 // [S x 256]
-    __nv_bfloat16 *DT = nullptr;                        // [256 x S]
-    float *loss = nullptr;
-    int32_t *draw_scene = nullptr, *pick = nullptr;  // [R], [R]
+    __nv_bfloat16 *D = nullptr;                         // [S x 256] per-scene sums of da1
+    BwPartials part{};                                  // the backward pass's partial sums
+    float *w2part = nullptr;                            // [kBwSplit x 256 x 256]
     float *zsel = nullptr;                           // [R x 8]
     float *hgb = nullptr;                            // [S x 256]: W1g grid + b1
-    int *status = nullptr;                           // fused kernel's error bits
+    int *status = nullptr;                           // error bits, 0 between calls
+    struct Report {                                  // pinned: what a call reads back
+        float loss;
+        int status;
+    } *report = nullptr;
+    float *loss = nullptr;
     int64_t adam_t = 0;
     int num_sms = 0;
     int forward_kernel = PIRRT_MLP_FORWARD_TCGEN05;
@@ -95,63 +99,49 @@ pirrt_status refresh_bf16(pirrt_proposal *P) {
     return PIRRT_OK;
 }
 
-// Grid part of layer 1 for the scenes: hg = grid W1g^T (BF16 in, FP32 out).
+// Grid part of layer 1 for the scenes: hg = grid W1g^T and hgb = hg + b1.
 pirrt_status scene_features(pirrt_proposal *P, int n_scenes, const float *grids) {
     if (n_scenes < 1 || n_scenes > P->max_scenes) return PIRRT_ERR_CAPACITY;
-    const int Sp = pad64(n_scenes);
-    PCK(cudaMemsetAsync(P->gridb, 0, sizeof(__nv_bfloat16) * (size_t)Sp * kGrid, P->stream));
-    PCK(cudaMemsetAsync(P->gridT, 0, sizeof(__nv_bfloat16) * (size_t)kGrid * Sp, P->stream));
-    to_bf16<<<blocks_for((int64_t)n_scenes * kGrid), 256, 0, P->stream>>>(
-        n_scenes, kGrid, grids, kGrid, P->gridb, kGrid, P->gridT, Sp);
+    scene_features_kernel<<<dim3(kHidden / kSceneN, (n_scenes + kSceneM - 1) / kSceneM), 128, kSceneSmem,
+                            P->stream>>>(n_scenes, grids, P->W1gb, P->w + ob1, P->hg, P->hgb);
     PCK(cudaGetLastError());
-    return gemm(P, Sp, kHidden, kGrid, P->gridb, kGrid, P->W1gb, kGrid, P->hg, kHidden, 0);
+    return PIRRT_OK;
 }
 
 // Rows through the network (after scene_features): y for `rows` samples.
-pirrt_status forward_rows(pirrt_proposal *P, int rows, const int32_t *scene, const float *z) {
+pirrt_status forward_rows(pirrt_proposal *P, int rows, const int32_t *scene, int rows_per_scene,
+                          const float *z) {
     if (rows < 1 || rows > P->max_rows) return PIRRT_ERR_CAPACITY;
     const int Rp = pad64(rows);
     layer1_rows<<<blocks_for((int64_t)Rp * kHidden), 256, 0, P->stream>>>(
-        rows, Rp, P->hg, scene, z, P->w + oW1n, P->w + ob1, P->a1, P->h1, P->h1T);
+        rows, Rp, P->hg, scene, rows_per_scene, z, P->w + oW1n, P->w + ob1, P->a1, P->h1);
     PCK(cudaGetLastError());
     pirrt_status rc = gemm(P, Rp, kHidden, kHidden, P->h1, kHidden, P->W2b, kHidden, P->a2, kHidden, 0);
     if (rc) return rc;
     bias_relu<<<blocks_for((int64_t)Rp * kHidden), 256, 0, P->stream>>>(rows, Rp, P->a2, P->w + ob2,
-                                                                         P->h2, nullptr);
+                                                                         P->h2);
     layer3_rows<<<blocks_for((int64_t)rows * 32), 256, 0, P->stream>>>(rows, P->h2, P->W3b,
                                                                         P->w + ob3, P->y);
     PCK(cudaGetLastError());
     return PIRRT_OK;
 }
 
-// hgb[s][j] = hg[s][j] + b1[j]: the per-scene part of layer 1 (the first
-// addition of the layered path's layer-1 sum, in the same order)
-__global__ void scene_bias(int n_scenes, const float *__restrict__ hg, const float *__restrict__ b1,
-                           float *__restrict__ hgb) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_scenes * kHidden;
-         i += gridDim.x * blockDim.x)
-        hgb[i] = hg[i] + b1[i % kHidden];
-}
-
 // The fused tcgen05 forward pass over `rows` rows (after scene_features):
 // y and / or the mixture `out` (see tc::FwdArgs).  The error bits are read
 // after the caller's stream synchronisation (read_status).
 pirrt_status forward_fused(pirrt_proposal *P, int n_scenes, int rows, const int32_t *scene,
-                           const float *z, float *y, const float *uniform_xy, const float *coin,
-                           float frac, float *out) {
+                           int rows_per_scene, const float *z, float *y, const float *uniform_xy,
+                           const float *coin, float frac, float *out) {
     if (rows < 1 || rows > P->max_rows) return PIRRT_ERR_CAPACITY;
     if (reinterpret_cast<uintptr_t>(z) % 16 || reinterpret_cast<uintptr_t>(y) % 8 ||
         reinterpret_cast<uintptr_t>(out) % 8 || reinterpret_cast<uintptr_t>(uniform_xy) % 8)
         return PIRRT_ERR_INVALID_ARG;
-    PCK(cudaMemsetAsync(P->status, 0, sizeof(int), P->stream));
-    scene_bias<<<blocks_for((int64_t)n_scenes * kHidden), 256, 0, P->stream>>>(n_scenes, P->hg,
-                                                                              P->w + ob1, P->hgb);
-    PCK(cudaGetLastError());
     tc::FwdArgs a{};
     a.rows = rows;
     a.n_scenes = n_scenes;
     a.hgb = P->hgb;
     a.scene = scene;
+    a.rows_per_scene = rows_per_scene;
     a.z = z;
     a.W1n = P->w + oW1n;
     a.W2b = P->W2b;
@@ -178,26 +168,27 @@ pirrt_status forward_fused(pirrt_proposal *P, int n_scenes, int rows, const int3
     return PIRRT_OK;
 }
 
-// Error bits of the last fused pass (call after a stream synchronisation).
-pirrt_status read_status(pirrt_proposal *P) {
-    int st = 0;
-    PCK(cudaMemcpy(&st, P->status, sizeof(int), cudaMemcpyDeviceToHost));
-    if (st & tc::kErrTimeout) return PIRRT_ERR_DEVICE_TIMEOUT;
-    if (st & tc::kErrScene) return PIRRT_ERR_BAD_INPUT;
-    return PIRRT_OK;
+// The end of a call: the error bits (and, with `loss`, the loss) come back with
+// one small copy ordered on the stream, and the call waits for it.
+pirrt_status finish_call(pirrt_proposal *P) {
+    PCK(cudaMemcpyAsync(P->report, P->loss, sizeof(*P->report), cudaMemcpyDeviceToHost, P->stream));
+    PCK(cudaStreamSynchronize(P->stream));
+    const int st = P->report->status;
+    if (st == 0) return PIRRT_OK;
+    PCK(cudaMemsetAsync(P->status, 0, sizeof(int), P->stream));
+    return st & tc::kErrTimeout ? PIRRT_ERR_DEVICE_TIMEOUT : PIRRT_ERR_BAD_INPUT;
 }
 
 // The forward pass of `rows` rows by the selected kernel into y (P->y if
 // null); a mixture into `out` when given.
 pirrt_status forward_any(pirrt_proposal *P, int n_scenes, int rows, const int32_t *scene,
-                         const float *z, float *y, const float *uniform_xy, const float *coin,
-                         float frac, float *out) {
+                         int rows_per_scene, const float *z, float *y, const float *uniform_xy,
+                         const float *coin, float frac, float *out) {
     if (P->forward_kernel == PIRRT_MLP_FORWARD_TCGEN05)
-        return forward_fused(P, n_scenes, rows, scene, z, y ? y : P->y, uniform_xy, coin, frac,
-                             out);
-    pirrt_status rc = forward_rows(P, rows, scene, z);
+        return forward_fused(P, n_scenes, rows, scene, rows_per_scene, z, y ? y : P->y, uniform_xy,
+                             coin, frac, out);
+    pirrt_status rc = forward_rows(P, rows, scene, rows_per_scene, z);
     if (rc) return rc;
-    PCK(cudaMemsetAsync(P->status, 0, sizeof(int), P->stream));
     P->last_rows = rows;
     P->last_has_acts = 1;
     if (y && y != P->y)
@@ -211,12 +202,13 @@ pirrt_status forward_any(pirrt_proposal *P, int n_scenes, int rows, const int32_
 }
 
 void free_all(pirrt_proposal *P) {
-    void *bufs[] = {P->w, P->m, P->v, P->grad, P->W1gb, P->W2b, P->W2Tb, P->W3b, P->gridb,
-                    P->gridT, P->hg, P->a1, P->a2, P->dh1, P->da2f, P->h1, P->h1T, P->h2,
-                    P->da2b, P->da2T, P->y, P->D, P->DT, P->loss, P->draw_scene, P->pick, P->zsel,
-                    P->hgb, P->status};
+    void *bufs[] = {P->w, P->m, P->v, P->grad, P->W1gb, P->W2b, P->W2Tb, P->W3b, P->hg, P->a1, P->a2,
+                    P->h1, P->h2, P->da2, P->y, P->D, P->loss, P->zsel, P->hgb, P->w2part,
+                    P->part.w3, P->part.b2, P->part.w1n, P->part.b1, P->part.tail, P->part.run,
+                    P->part.run_scene};
     for (void *b : bufs)
         if (b) cudaFree(b);
+    if (P->report) cudaFreeHost(P->report);
     for (cudaEvent_t &e : P->kev)
         if (e) cudaEventDestroy(e);
 }
@@ -272,32 +264,38 @@ pirrt_status pirrt_proposal_create(int32_t max_scenes, int32_t max_rows, uint64_
     PA(P->W2b, bf * nW2);
     PA(P->W2Tb, bf * nW2);
     PA(P->W3b, bf * nW3);
-    PA(P->gridb, bf * S * kGrid);
-    PA(P->gridT, bf * S * kGrid);
     PA(P->hg, f * S * kHidden);
     PA(P->a1, f * R * kHidden);
     PA(P->a2, f * R * kHidden);
-    PA(P->dh1, f * R * kHidden);
-    PA(P->da2f, f * R * kHidden);
     PA(P->h1, bf * R * kHidden);
-    PA(P->h1T, bf * R * kHidden);
     PA(P->h2, bf * R * kHidden);
-    PA(P->da2b, bf * R * kHidden);
-    PA(P->da2T, bf * R * kHidden);
+    PA(P->da2, bf * R * kHidden);
     PA(P->y, f * R * kOut);
-    PA(P->D, f * S * kHidden);
-    PA(P->DT, bf * S * kHidden);
-    PA(P->loss, f * 4);
-    PA(P->draw_scene, sizeof(int32_t) * R);
-    PA(P->pick, sizeof(int32_t) * R);
+    PA(P->D, bf * S * kHidden);
     PA(P->zsel, f * R * kNoise);
     PA(P->hgb, f * S * kHidden);
-    PA(P->status, sizeof(int));
+    PA(P->loss, sizeof(pirrt_proposal::Report));  // the loss, then the error bits
+    P->status = reinterpret_cast<int *>(P->loss + 1);
+    if (cudaDeviceGetAttribute(&P->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+        return bail(PIRRT_ERR_CUDA);
+    const size_t C = (size_t)P->num_sms;  // CTAs of the backward pass, at most
+    PA(P->part.w3, f * C * kOut * kHidden);
+    PA(P->part.b2, f * C * kHidden);
+    PA(P->part.w1n, f * C * kHidden * kNoise);
+    PA(P->part.b1, f * C * kHidden);
+    PA(P->part.tail, f * C * 4);
+    PA(P->part.run, f * R * kHidden);
+    PA(P->part.run_scene, sizeof(int) * R);
+    PA(P->w2part, f * kBwSplit * kHidden * kHidden);
 #undef PA
     if (cudaEventCreate(&P->kev[0]) != cudaSuccess || cudaEventCreate(&P->kev[1]) != cudaSuccess ||
-        cudaDeviceGetAttribute(&P->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaMallocHost((void **)&P->report, sizeof(*P->report)) != cudaSuccess ||
+        cudaFuncSetAttribute(backward_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(BwShared)) != cudaSuccess ||
         cudaFuncSetAttribute(tc::mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc::kSmemBytes) != cudaSuccess) {
+                             tc::kSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(scene_features_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kSceneSmem) != cudaSuccess) {
         cudaGetLastError();
         return bail(PIRRT_ERR_CUDA);
     }
@@ -363,11 +361,10 @@ pirrt_status pirrt_proposal_forward(pirrt_proposal *P, int32_t n_scenes, const f
     PCK(cudaSetDevice(P->device));
     pirrt_status rc = scene_features(P, n_scenes, grids);
     if (rc) return rc;
-    if ((rc = forward_any(P, n_scenes, rows, scene, noise, out_xy, nullptr, nullptr, 0.f,
+    if ((rc = forward_any(P, n_scenes, rows, scene, 1, noise, out_xy, nullptr, nullptr, 0.f,
                           nullptr)))
         return rc;
-    PCK(cudaStreamSynchronize(P->stream));
-    return read_status(P);
+    return finish_call(P);
 }
 
 pirrt_status pirrt_proposal_sample(pirrt_proposal *P, int32_t n_scenes, const float *grids,
@@ -380,11 +377,10 @@ pirrt_status pirrt_proposal_sample(pirrt_proposal *P, int32_t n_scenes, const fl
     PCK(cudaSetDevice(P->device));
     pirrt_status rc = scene_features(P, n_scenes, grids);
     if (rc) return rc;
-    if ((rc = forward_any(P, n_scenes, rows, scene, noise, nullptr, uniform_xy, coin,
+    if ((rc = forward_any(P, n_scenes, rows, scene, 1, noise, nullptr, uniform_xy, coin,
                           learned_fraction, out_xy)))
         return rc;
-    PCK(cudaStreamSynchronize(P->stream));
-    return read_status(P);
+    return finish_call(P);
 }
 
 pirrt_status pirrt_proposal_imle_select(pirrt_proposal *P, int32_t n_scenes, const float *grids,
@@ -397,14 +393,98 @@ pirrt_status pirrt_proposal_imle_select(pirrt_proposal *P, int32_t n_scenes, con
     if ((int64_t)n_targets * K > P->max_rows) return PIRRT_ERR_CAPACITY;
     pirrt_status rc = scene_features(P, n_scenes, grids);
     if (rc) return rc;
-    if ((rc = forward_any(P, n_scenes, n_targets * K, draw_scene, noise, nullptr, nullptr, nullptr,
+    if ((rc = forward_any(P, n_scenes, n_targets * K, draw_scene, 1, noise, nullptr, nullptr, nullptr,
                           0.f, nullptr)))
         return rc;
     imle_select<<<blocks_for(n_targets), 256, 0, P->stream>>>(n_targets, K, P->y, targets, pick);
     PCK(cudaGetLastError());
-    PCK(cudaStreamSynchronize(P->stream));
-    return read_status(P);
+    return finish_call(P);
 }
+
+extern "C++" {
+// The backward pass of `rows` rows (after scene_features); the loss stays on the
+// device (finish_call reads it).
+static pirrt_status backward_rows(pirrt_proposal *P, int n_scenes, const float *grids, int rows,
+                                  const int32_t *scene, const float *noise, const float *targets) {
+    if (rows < 1 || rows > P->max_rows) return PIRRT_ERR_CAPACITY;
+    P->last_rows = rows;
+    P->last_has_acts = 1;
+    BwArgs a{};
+    a.rows = rows;
+    a.tiles = pad64(rows) / kBwRows;
+    // a CTA's share of the tiles: one each while they last, so that every SM works
+    const int most = a.tiles < P->num_sms ? a.tiles : P->num_sms;
+    a.tiles_per_cta = (a.tiles + most - 1) / most;
+    const int ctas = (a.tiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
+    a.n_scenes = n_scenes;
+    a.hg = P->hg;
+    a.b1 = P->w + ob1;
+    a.b2 = P->w + ob2;
+    a.b3 = P->w + ob3;
+    a.W1n = P->w + oW1n;
+    a.W2b = P->W2b;
+    a.W2Tb = P->W2Tb;
+    a.W3b = P->W3b;
+    a.scene = scene;
+    a.z = noise;
+    a.target = targets;
+    a.h1 = P->h1;
+    a.h2 = P->h2;
+    a.da2 = P->da2;
+    a.y = P->y;
+    a.part = P->part;
+    a.status = P->status;
+    backward_rows_kernel<<<ctas, kBwThreads, sizeof(BwShared), P->stream>>>(a);
+    PCK(cudaGetLastError());
+    // dW2 in parts of at least 128 rows, so that 16 tiles of 64 x 64 become up to
+    // 256 CTAs
+    const int rows_pad = a.tiles * kBwRows;
+    int splits = (rows_pad + 127) / 128;
+    if (splits > kBwSplit) splits = kBwSplit;
+    const int per = ((rows_pad + splits - 1) / splits + 31) / 32 * 32;
+    splits = (rows_pad + per - 1) / per;
+    dw2_parts_kernel<<<dim3(4, 4, splits), 128, 0, P->stream>>>(rows_pad, per, P->da2, P->h1,
+                                                               P->w2part);
+    finish_backward_kernel<<<kFinishRow + kFinishSmall + n_scenes, 256, 0, P->stream>>>(
+        ctas, splits, rows_pad, rows, P->part, P->w2part, P->grad + oW2, P->grad + oW3,
+        P->grad + ob2, P->grad + ob3, P->grad + oW1n, P->grad + ob1, P->loss, P->D);
+    dw1g_kernel<<<dim3(kHidden / 64, kGrid / 64), 128, 0, P->stream>>>(n_scenes, P->D, grids,
+                                                                      P->grad + oW1g);
+    PCK(cudaGetLastError());
+    return PIRRT_OK;
+}
+
+// One Adam step for the t-th time; with `status` it is skipped if an earlier
+// kernel of the call reported an error.
+static pirrt_status adam_all(pirrt_proposal *P, int64_t t, float lr, float beta1, float beta2,
+                             float eps, const int *status) {
+    AdamArgs a{};
+    a.w = P->w;
+    a.m = P->m;
+    a.v = P->v;
+    a.grad = P->grad;
+    a.W1gb = P->W1gb;
+    a.W2b = P->W2b;
+    a.W2Tb = P->W2Tb;
+    a.W3b = P->W3b;
+    a.n = kParams;
+    a.oW2 = oW2;
+    a.ob2 = ob2;
+    a.oW3 = oW3;
+    a.ob3 = ob3;
+    a.nW1g = nW1g;
+    a.lr = lr;
+    a.beta1 = beta1;
+    a.beta2 = beta2;
+    a.eps = eps;
+    a.bc1 = 1.f - std::pow(beta1, (float)t);
+    a.bc2 = 1.f - std::pow(beta2, (float)t);
+    a.status = status;
+    adam_all_kernel<<<(unsigned)((kParams + 255) / 256), 256, 0, P->stream>>>(a);
+    PCK(cudaGetLastError());
+    return PIRRT_OK;
+}
+}  // extern "C++"
 
 pirrt_status pirrt_proposal_backward(pirrt_proposal *P, int32_t n_scenes, const float *grids,
                                      int32_t rows, const int32_t *scene, const float *noise,
@@ -413,58 +493,18 @@ pirrt_status pirrt_proposal_backward(pirrt_proposal *P, int32_t n_scenes, const 
     PCK(cudaSetDevice(P->device));
     pirrt_status rc = scene_features(P, n_scenes, grids);
     if (rc) return rc;
-    if ((rc = forward_rows(P, rows, scene, noise))) return rc;
-    P->last_rows = rows;
-    P->last_has_acts = 1;
-    const int Rp = pad64(rows), Sp = pad64(n_scenes);
-    output_backward<<<kHidden, 256, 0, P->stream>>>(rows, Rp, P->y, targets, P->h2, P->W3b, P->a2,
-                                                   P->grad + oW3, P->grad + ob3, P->da2b, P->da2T,
-                                                   P->da2f, P->loss);
-    PCK(cudaGetLastError());
-    // dW2 += da2^T h1 ; db2 += sum da2 ; dh1 = da2 W2
-    if ((rc = gemm(P, kHidden, kHidden, Rp, P->da2T, Rp, P->h1T, Rp, P->grad + oW2, kHidden, 1)))
-        return rc;
-    col_sum<<<1, kHidden, 0, P->stream>>>(rows, kHidden, P->da2f, P->grad + ob2);
-    if ((rc = gemm(P, Rp, kHidden, kHidden, P->da2b, kHidden, P->W2Tb, kHidden, P->dh1, kHidden, 0)))
-        return rc;
-    // da1 = dh1 masked by relu(a1): per-scene sums D, dW1n, db1
-    PCK(cudaMemsetAsync(P->D, 0, sizeof(float) * (size_t)Sp * kHidden, P->stream));
-    layer1_backward<<<1, kHidden, 0, P->stream>>>(rows, P->dh1, P->a1, scene, noise, P->D,
-                                                  P->grad + oW1n, P->grad + ob1);
-    PCK(cudaGetLastError());
-    // dW1g += D^T grid (BF16 D, transposed)
-    PCK(cudaMemsetAsync(P->DT, 0, sizeof(__nv_bfloat16) * (size_t)Sp * kHidden, P->stream));
-    to_bf16<<<blocks_for((int64_t)n_scenes * kHidden), 256, 0, P->stream>>>(
-        n_scenes, kHidden, P->D, kHidden, nullptr, 0, P->DT, Sp);
-    PCK(cudaGetLastError());
-    if ((rc = gemm(P, kHidden, kGrid, Sp, P->DT, Sp, P->gridT, Sp, P->grad + oW1g, kGrid, 1)))
-        return rc;
-    if (loss_out) PCK(cudaMemcpyAsync(loss_out, P->loss, sizeof(float), cudaMemcpyDeviceToHost,
-                                      P->stream));
-    PCK(cudaStreamSynchronize(P->stream));
-    return PIRRT_OK;
+    if ((rc = backward_rows(P, n_scenes, grids, rows, scene, noise, targets))) return rc;
+    rc = finish_call(P);
+    if (loss_out) *loss_out = P->report->loss;
+    return rc;
 }
 
 pirrt_status pirrt_proposal_adam(pirrt_proposal *P, float lr, float beta1, float beta2, float eps) {
     if (!P || !(lr > 0.f)) return PIRRT_ERR_INVALID_ARG;
     PCK(cudaSetDevice(P->device));
     P->adam_t += 1;
-    const float bc1 = 1.f - std::pow(beta1, (float)P->adam_t);
-    const float bc2 = 1.f - std::pow(beta2, (float)P->adam_t);
-    struct Seg { int64_t off; int rows, cols; __nv_bfloat16 *b, *bT; int ldT; };
-    const Seg segs[] = {{oW1g, kHidden, kGrid, P->W1gb, nullptr, 0},
-                        {oW1n, kHidden, kNoise, nullptr, nullptr, 0},
-                        {ob1, 1, kHidden, nullptr, nullptr, 0},
-                        {oW2, kHidden, kHidden, P->W2b, P->W2Tb, kHidden},
-                        {ob2, 1, kHidden, nullptr, nullptr, 0},
-                        {oW3, kOut, kHidden, P->W3b, nullptr, 0},
-                        {ob3, 1, kOut, nullptr, nullptr, 0}};
-    for (const Seg &g : segs) {
-        adam_step<<<blocks_for((int64_t)g.rows * g.cols), 256, 0, P->stream>>>(
-            g.rows, g.cols, P->w + g.off, P->m + g.off, P->v + g.off, P->grad + g.off, lr, beta1,
-            beta2, eps, bc1, bc2, g.b, g.bT, g.ldT);
-    }
-    PCK(cudaGetLastError());
+    const pirrt_status rc = adam_all(P, P->adam_t, lr, beta1, beta2, eps, nullptr);
+    if (rc) return rc;
     PCK(cudaStreamSynchronize(P->stream));
     return PIRRT_OK;
 }
@@ -477,25 +517,26 @@ pirrt_status pirrt_proposal_train_step(pirrt_proposal *P, int32_t n_scenes, cons
         return PIRRT_ERR_INVALID_ARG;
     if ((int64_t)n_targets * K > P->max_rows) return PIRRT_ERR_CAPACITY;
     PCK(cudaSetDevice(P->device));
-    repeat_scene<<<blocks_for((int64_t)n_targets * K), 256, 0, P->stream>>>(n_targets, K,
-                                                                           target_scene,
-                                                                           P->draw_scene);
-    PCK(cudaGetLastError());
     pirrt_status rc = scene_features(P, n_scenes, grids);
     if (rc) return rc;
-    if ((rc = forward_any(P, n_scenes, n_targets * K, P->draw_scene, noise, nullptr, nullptr,
+    // the draws (row t*K + k in target t's scene), the nearest of each target, its
+    // backward pass and Adam, with one wait at the end
+    if ((rc = forward_any(P, n_scenes, n_targets * K, target_scene, K, noise, nullptr, nullptr,
                           nullptr, 0.f, nullptr)))
         return rc;
-    imle_select<<<blocks_for(n_targets), 256, 0, P->stream>>>(n_targets, K, P->y, targets, P->pick);
-    gather_noise<<<blocks_for((int64_t)n_targets * kNoise), 256, 0, P->stream>>>(n_targets, K, noise,
-                                                                                P->pick, P->zsel);
+    select_noise_kernel<<<(n_targets * 8 + 255) / 256, 256, 0, P->stream>>>(n_targets, K, P->y, targets,
+                                                                          noise, P->zsel);
     PCK(cudaGetLastError());
-    if ((rc = pirrt_proposal_backward(P, n_scenes, grids, n_targets, target_scene, P->zsel, targets,
-                                      loss_out)))
+    if ((rc = backward_rows(P, n_scenes, grids, n_targets, target_scene, P->zsel, targets)))
         return rc;
-    // the selection pass's error bits (the backward pass synchronised)
-    if ((rc = read_status(P))) return rc;
-    return pirrt_proposal_adam(P, lr, 0.9f, 0.999f, 1e-8f);
+    const bool step = lr > 0.f;
+    if (step && (rc = adam_all(P, P->adam_t + 1, lr, 0.9f, 0.999f, 1e-8f, P->status))) return rc;
+    rc = finish_call(P);
+    if (loss_out) *loss_out = P->report->loss;
+    if (rc) return rc;
+    if (!step) return PIRRT_ERR_INVALID_ARG;
+    P->adam_t += 1;
+    return PIRRT_OK;
 }
 
 pirrt_status pirrt_proposal_set_options(pirrt_proposal *P, int32_t forward_kernel,
