@@ -132,16 +132,16 @@ def edges(points, nbr, scene: Scene, exact_segment: bool, n_check: int = 16,
     tdt = torch.float64 if f64 else torch.float32
     start = torch.empty(n + 1, dtype=torch.int64, device="cuda")
     m = ctypes.c_int64(0)
-    args = (dim, n, points.data_ptr(), k, nbr.data_ptr(), len(scene.radii), c.data_ptr(),
-            r.data_ptr(), 0 if exact_segment else 1, int(n_check), 1 if f64 else 0)
-    rc = lib.rgg_edges(*args, None, None, None, start.data_ptr(), 0, ctypes.byref(m), _stream())
-    if rc not in (0, 3):
-        _check("rgg_edges", rc)
-    cap = int(m.value)
-    u = torch.empty(max(cap, 1), dtype=torch.int32, device="cuda")
-    v = torch.empty(max(cap, 1), dtype=torch.int32, device="cuda")
-    cost = torch.empty(max(cap, 1), dtype=tdt, device="cuda")
-    _check("rgg_edges", lib.rgg_edges(*args, u.data_ptr(), v.data_ptr(), cost.data_ptr(),
+    # room for every link (a second pass over the links to count them first would
+    # cost as much as the first); the result is a view of its used part
+    cap = n * k
+    u = torch.empty(cap, dtype=torch.int32, device="cuda")
+    v = torch.empty(cap, dtype=torch.int32, device="cuda")
+    cost = torch.empty(cap, dtype=tdt, device="cuda")
+    _check("rgg_edges", lib.rgg_edges(dim, n, points.data_ptr(), k, nbr.data_ptr(),
+                                      len(scene.radii), c.data_ptr(), r.data_ptr(),
+                                      0 if exact_segment else 1, int(n_check), 1 if f64 else 0,
+                                      u.data_ptr(), v.data_ptr(), cost.data_ptr(),
                                       start.data_ptr(), cap, ctypes.byref(m), _stream()))
     mm = int(m.value)
     return u[:mm], v[:mm], cost[:mm], start.cpu().numpy()
