@@ -367,8 +367,8 @@ int64_t pirrt_graph_get_trace(const pirrt_graph *g, pirrt_trace_record *out, int
  * service for callers that cannot call cudaMalloc when they need g -- a
  * real-time planning loop that fixes all of its memory at start-up and must
  * not stall on, or fail in, the allocator in the middle of a control cycle.
- * It computes g(v) = g(parent(v)) + parent_cost[v] from the root by the same
- * pointer-jumping kernel as the graph handle, FP64 throughout:
+ * It computes g(v) = g(parent(v)) + parent_cost[v] from the root by pointer
+ * jumping in one kernel launch, FP64 throughout:
  *   n            vertex count, at most 262,144 (PIRRT_ERR_CAPACITY beyond)
  *   root         vertex with g = 0 (its parent entry is ignored)
  *   parent       device int32[n]: parent id in [0, n), or -1 for unreached
@@ -381,13 +381,13 @@ int64_t pirrt_graph_get_trace(const pirrt_graph *g, pirrt_trace_record *out, int
  * before the evaluation follows it: a parent id outside [0, n) other than -1,
  * or a bad cost, gives PIRRT_ERR_BAD_INPUT with g_out holding only the
  * initial values (0 at the root, +inf elsewhere).  Scratch lives in one
- * file-scope device array of about 11.5 MB that every GPU loading the library
+ * file-scope device array of about 8.4 MB that every GPU loading the library
  * holds until the process exits.  The first call on a device (with that
- * device current) resolves the array's device address and the launch shape.
- * Every call shares the array and clears what it needs, so calls that
- * overlap on the GPU (other streams, other host threads) race: serialise
- * them.  The call reads its status word back and synchronises the stream
- * before it returns.  Errors: PIRRT_ERR_INVALID_ARG, PIRRT_ERR_CAPACITY,
+ * device current) resolves the array's device address and the launch shape
+ * and pins one static page of host memory, where the kernel leaves its
+ * outcome.  Every call shares the array, so calls that overlap on the GPU
+ * (other streams, other host threads) race: serialise them.  The call
+ * synchronises the stream before it returns.  Errors: PIRRT_ERR_INVALID_ARG, PIRRT_ERR_CAPACITY,
  * PIRRT_ERR_BAD_INPUT, PIRRT_ERR_BAD_TREE (a cycle: the pointer-jumping round
  * limit ends the kernel), PIRRT_ERR_DEVICE_TIMEOUT, PIRRT_ERR_CUDA. */
 pirrt_status pirrt_evaluate_noalloc(int64_t n, int32_t root, const int32_t *parent,
