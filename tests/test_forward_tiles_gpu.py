@@ -1,7 +1,9 @@
 """The fused forward pass where its tiles end (128 rows, one to four tiles per CTA
-of 152), against the layered kernels with the bounds of test_mlp_gpu, and the
-same rows in another order: a row's arithmetic does not depend on the tile, the
-lane or the neighbours it lands on, so its result is the same bit for bit."""
+of 152): against the oracle on dyadic inputs (whose layer sums are exact in FP32,
+so that rounding cancellations cannot enter) with the bounds derived in
+test_mlp_gpu, and the same rows in another order -- a row's arithmetic does not
+depend on the tile, the lane or the neighbours it lands on, so its result is the
+same bit for bit."""
 import numpy as np
 import pytest
 
@@ -16,7 +18,15 @@ torch = T.torch
 @pytest.mark.parametrize("rows", [31, 127, 129, 152 * 128 - 1, 152 * 128, 152 * 128 + 1,
                                   152 * 128 * 3 + 65])
 def test_tile_edges(torch, rows):
-    T.test_fused_forward_matches_layered(torch, rows)
+    S = 6
+    params, grids, scene, z, target = T._dyadic(seed=rows, S=S, R=rows)
+    prop = P.Proposal(S, rows, seed=3)
+    gd, sd, zd, _ = T._upload(torch, prop, params, grids, scene, z, target)
+    y = prop.forward(gd, sd, zd).cpu().numpy().astype(np.float64)
+    f = M.forward(params, grids, scene, z.astype(np.float64), rounded=True)
+    atol = 0.25 * T.ACC * (f["h2"] @ np.abs(params["W3"]).T) + 2.0 ** -21
+    assert not (np.abs(y - f["y"]) > 1e-5 * np.abs(f["y"]) + atol).any()
+    prop.close()
 
 
 @pytest.mark.parametrize("S,rows", [(1, 300), (40, 129), (40, 152 * 128 + 513)])
