@@ -518,7 +518,7 @@ KERNEL_FILES = {"improve": ("improve_push.cuh", "improve_screen.cuh", "graph_ker
                             "replan_iteration.cuh", "replan_loop.cuh", "device_common.cuh"),
                 "evaluate": ("graph_kernels.cuh", "replan_iteration.cuh", "replan_loop.cuh",
                              "improve_push.cuh", "evaluate_async.cuh", "device_common.cuh"),
-                "insert": ("graph_kernels.cuh", "device_common.cuh")}
+                "insert": ("insert.cuh", "graph_kernels.cuh", "device_common.cuh")}
 
 
 def kernel_hash(kernel: str) -> str:

@@ -31,40 +31,6 @@ __device__ __forceinline__ void offer(unsigned long long *cand, int32_t v, doubl
 // Insertion
 // ---------------------------------------------------------------------------
 
-// Validate the new undirected edges and count, per endpoint, how many CSR
-// entries the block adds.  Invalid input raises kStatusBadInput and is not
-// counted (the host then discards the whole block).
-template <typename CT>
-__global__ void __launch_bounds__(kThreads)
-insert_validate_count(int64_t n_edges, const int32_t *__restrict__ src,
-                      const int32_t *__restrict__ dst, const CT *__restrict__ cost,
-                      int64_t n_old, int64_t n_after, int32_t *__restrict__ deg,
-                      int32_t *__restrict__ touched, DevCounters *ctr) {
-    // an old row gaining its first new entry joins the touched list (the new
-    // rows [n_old, n_after) are handled as a range)
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < n_edges;
-         base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = base + threadIdx.x;
-        bool ta = false, tb = false;
-        int32_t a = 0, b = 0;
-        if (e < n_edges) {
-            a = src[e];
-            b = dst[e];
-            const double c = (double)cost[e];
-            const bool ok = a >= 0 && b >= 0 && a < n_after && b < n_after && a != b &&
-                            c > 0.0 && c <= DBL_MAX;  // rejects NaN, +inf, <= 0
-            if (!ok) {
-                atomicOr(&ctr->status, kStatusBadInput);
-            } else {
-                ta = atomicAdd(&deg[a], 1) == 0 && a < n_old;
-                tb = atomicAdd(&deg[b], 1) == 0 && b < n_old;
-            }
-        }
-        warp_append(ta, a, touched, &ctr->n_touched);
-        warp_append(tb, b, touched, &ctr->n_touched);
-    }
-}
-
 // Room a moving row reserves: 1.5x its new length + 4 (a few moves over a
 // row's life); a repacked row gets 1.25x + 2, so a repack always fits a pool
 // of 2 x (directed entries) + 4 x (vertices).
@@ -154,105 +120,6 @@ scan_tile_apply(const int32_t *__restrict__ deg, int64_t len,
         if (x < len) new_off[x] = run;
         run += v[i];
     }
-}
-
-// Start of an insertion: empty touched list, no room taken, no error.
-static __global__ void insert_begin_kernel(DevCounters *c) {
-    c->n_touched = 0u;
-    c->pool_cursor = 0ull;
-    c->status = 0u;
-}
-
-// Item k of the rows an insertion changes: the touched old rows, then the new
-// rows [n_old, n_after).
-__device__ __forceinline__ int64_t changed_row(int64_t k, int64_t nt, const int32_t *touched,
-                                               int64_t n_old) {
-    return k < nt ? (int64_t)touched[k] : n_old + (k - nt);
-}
-
-// Plan without a scan: a changed row that would overflow (every new row with
-// entries) takes room at the end of the pool from a cursor, one atomic per
-// block; pool offsets (relative to the cursor's base) go to off[v].  Rows
-// keep their relative order within a block only, which nothing relies on.
-static __global__ void __launch_bounds__(kThreads)
-insert_plan_list(int64_t n_old, int64_t n_after, const int32_t *__restrict__ touched,
-                 const RowExt *__restrict__ rows, const int32_t *__restrict__ deg,
-                 int32_t *__restrict__ alloc, int64_t *__restrict__ off, DevCounters *ctr) {
-    const int64_t nt = (int64_t)__ldcg(&ctr->n_touched);
-    const int64_t total = nt + (n_after - n_old);
-    __shared__ long long s_base;
-    for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < total;
-         base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = base + threadIdx.x;
-        int32_t a = 0;
-        int64_t v = -1;
-        if (k < total) {
-            v = changed_row(k, nt, touched, n_old);
-            const int32_t len = v < n_old ? rows[v].len : 0;
-            const int32_t cap = v < n_old ? rows[v].cap : 0;
-            const int32_t need = len + deg[v];
-            if (need > cap) a = row_room(need, false);
-            alloc[v] = a;
-        }
-        long long tot;
-        const long long ex = block_exclusive_scan(a, &tot);
-        if (threadIdx.x == 0)
-            s_base = tot ? (long long)atomicAdd(&ctr->pool_cursor, (unsigned long long)tot) : 0;
-        __syncthreads();
-        if (a > 0) off[v] = s_base + ex;
-        __syncthreads();
-    }
-}
-
-// Move the changed rows that took new room (their old entries first) to pool
-// offset base + off[v], and set every changed row's extent to its length
-// after the block.  One warp per 32 changed rows.
-template <typename CT>
-__global__ void __launch_bounds__(kThreads)
-insert_move_list(int64_t n_old, int64_t n_after, const int32_t *__restrict__ touched,
-                 RowExt *__restrict__ rows, const int32_t *__restrict__ deg,
-                 const int32_t *__restrict__ alloc, const int64_t *__restrict__ off,
-                 long long base, Entry<CT> *__restrict__ pool, DevCounters *ctr) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nt = (int64_t)__ldcg(&ctr->n_touched);
-    const int64_t total = nt + (n_after - n_old);
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    unsigned long long copied = 0;
-    for (int64_t w0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
-         w0 < total; w0 += warps * 32) {
-        const int64_t k = w0 + lane;
-        long long ob = 0, nb = 0;
-        int32_t len = 0;
-        bool move = false;
-        if (k < total) {
-            const int64_t v = changed_row(k, nt, touched, n_old);
-            RowExt r{0, 0, 0};
-            if (v < n_old) r = rows[v];
-            const int32_t a = alloc[v];
-            len = r.len;
-            ob = r.beg;
-            RowExt nr = r;
-            nr.len = r.len + deg[v];
-            if (a > 0) {
-                nb = base + off[v];
-                nr.beg = nb;
-                nr.cap = a;
-                move = len > 0;
-            }
-            rows[v] = nr;
-        }
-        unsigned todo = __ballot_sync(0xffffffffu, move);
-        while (todo) {
-            const int l = __ffs(todo) - 1;
-            todo &= todo - 1u;
-            const long long sb = __shfl_sync(0xffffffffu, ob, l);
-            const long long db = __shfl_sync(0xffffffffu, nb, l);
-            const int32_t n = __shfl_sync(0xffffffffu, len, l);
-            for (int32_t q = lane; q < n; q += 32) pool[db + q] = ld_stream(&pool[sb + q]);
-            copied += (unsigned long long)n;
-        }
-    }
-    if (lane == 0 && copied) atomicAdd(&ctr->insert_copied, copied);
 }
 
 // Slack CSR.  Every row owns adj[beg, beg + cap) of a pool and fills it from
@@ -365,82 +232,6 @@ export_rows(int64_t n, const RowExt *__restrict__ rows, const int64_t *__restric
             const long long d0 = __shfl_sync(0xffffffffu, db, l);
             const int32_t k0 = __shfl_sync(0xffffffffu, len, l);
             for (int32_t k = lane; k < k0; k += 32) out[d0 + k] = adj[s0 + k];
-        }
-    }
-}
-
-// Place both directions of every new edge at the tail of its rows (filled
-// from the row end, order within a row is irrelevant) and seed the next
-// Improve frontier with both endpoints.
-template <typename CT>
-__global__ void __launch_bounds__(kThreads)
-insert_scatter(int64_t n_edges, const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
-               const CT *__restrict__ cost, const RowExt *__restrict__ rows,
-               int32_t *__restrict__ deg, Entry<CT> *__restrict__ adj, unsigned *__restrict__ stamp,
-               int32_t root, int32_t *__restrict__ list0, int32_t *__restrict__ list1,
-               const double *__restrict__ g, unsigned long long *__restrict__ cand,
-               DevCounters *ctr) {
-    const unsigned epoch = ctr->epoch;
-    int32_t *active = (ctr->la & 1u) ? list1 : list0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n_edges; base += stride) {
-        const int64_t e = base + threadIdx.x;
-        bool pa = false, pb = false;
-        int32_t a = 0, b = 0;
-        if (e < n_edges) {
-            a = src[e];
-            b = dst[e];
-            const CT w = cost[e];
-            // rows hold the lengths after the block: fill the tails from the end
-            const int64_t sa = rows[a].beg + rows[a].len - atomicSub(&deg[a], 1);
-            const int64_t sb = rows[b].beg + rows[b].len - atomicSub(&deg[b], 1);
-            Entry<CT> ea{}, eb{};
-            ea.col = b;
-            ea.w = w;
-            eb.col = a;
-            eb.w = w;
-            adj[sa] = ea;
-            adj[sb] = eb;
-            // the new edge offers each endpoint the other's candidate; an
-            // endpoint joins the next Improve list only if that candidate beats
-            // its g (g >= cur, so a candidate not below g can never win; a new
-            // vertex has g = +inf and joins with its first finite neighbour)
-            const double ga = g[a], gb = g[b];
-            const double va = gb + widen(w), vb = ga + widen(w);
-            const bool ua = a != root && gb < CUDART_INF && va < ga;
-            const bool ub = b != root && ga < CUDART_INF && vb < gb;
-            if (ub) offer(cand, b, vb);
-            if (ua) offer(cand, a, va);
-            pa = ua && atomicExch(&stamp[a], epoch) != epoch;
-            pb = ub && atomicExch(&stamp[b], epoch) != epoch;
-        }
-        __shared__ unsigned long long s_scan[kThreads / 32 + 2];
-        unsigned ba, bb;
-        block_reserve2<kThreads>(pa ? 1u : 0u, pb ? 1u : 0u, &ctr->n_active, &ctr->n_active,
-                                 s_scan, ba, bb);
-        if (pa) active[ba] = a;
-        if (pb) active[bb] = b;
-    }
-}
-
-// Seed the new vertices: g = +inf (0 for the root), no parent, no offer.
-// They join the next Improve frontier through the offers of their new edges
-// (insert_scatter).
-template <typename CT>
-__global__ void __launch_bounds__(kThreads)
-insert_init_vertices(int64_t n_old, int64_t n_after, int32_t root, double *__restrict__ g,
-                     float *__restrict__ g32, int32_t *__restrict__ p, CT *__restrict__ pc,
-                     unsigned long long *__restrict__ cand, unsigned *__restrict__ stamp,
-                     int32_t *__restrict__ list0, int32_t *__restrict__ list1, DevCounters *ctr) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = n_old + (int64_t)blockIdx.x * blockDim.x; base < n_after; base += stride) {
-        const int64_t v = base + threadIdx.x;
-        if (v < n_after) {
-            g[v] = (v == root) ? 0.0 : CUDART_INF;
-            g32[v] = (v == root) ? 0.0f : __int_as_float(0x7f800000);
-            p[v] = (v == root) ? kRootMark : -1;
-            pc[v] = CT(0);
-            cand[v] = kCandNone;
         }
     }
 }

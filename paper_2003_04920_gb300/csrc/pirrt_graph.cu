@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -26,6 +27,7 @@
 #include "improve_screen.cuh"
 #include "improve_tma.cuh"
 #include "replan_iteration.cuh"
+#include "insert.cuh"
 #include "replan_loop.cuh"
 #include "pirrt.h"
 
@@ -63,6 +65,9 @@ struct pirrt_graph {
     int64_t *roff = nullptr;       // insertion / export: exclusive scan
     unsigned long long copied_seen = 0;
     int64_t *hx = nullptr;         // pinned host scalars read back by insertion
+    InsertReport *insert_rep = nullptr;  // pinned: what an insertion's kernel tells the host
+    unsigned insert_seq = 0;
+    int insert_blocks = 0;               // co-resident grid of the insertion kernel
     double *g = nullptr;
     float *g32 = nullptr;  // FP32 shadow of g for candidate screening
     int32_t *p = nullptr;
@@ -622,102 +627,117 @@ pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const i
                          const int32_t *dst, const CT *cost) {
     const int64_t n_old = G->n, n_after = G->n + n_new;
     const int64_t m_after = G->m + 2 * n_edges;
-    const int max_blocks = G->num_sms * 32;
     const bool prof = G->profiling != 0;
     if (prof) CK(cudaEventRecord(G->pev[6], G->stream));
-    // 1. validate and count new entries per row (deg is all zero between
-    //    insertions: the scatter below takes every count back); the old rows
-    //    gaining entries form the touched list
-    insert_begin_kernel<<<1, 1, 0, G->stream>>>(G->ctr);
-    CKL();
-    if (n_edges > 0) {
-        insert_validate_count<CT><<<grid_for(n_edges, kThreads, max_blocks), kThreads, 0, G->stream>>>(
-            n_edges, src, dst, cost, n_old, n_after, G->deg, G->touched, G->ctr);
-        CKL();
-    }
-    // 2. room at the end of the pool for the changed rows that would overflow,
-    //    from a cursor (no scan over every row); one host read of the
-    //    validation status and the room taken
-    const int64_t changed_max = std::min<int64_t>(2 * n_edges, n_old) + n_new;
-    if (changed_max > 0) {
-        insert_plan_list<<<grid_for(changed_max, kThreads, max_blocks), kThreads, 0, G->stream>>>(
-            n_old, n_after, G->touched, G->rows, G->deg, G->ralloc, G->roff, G->ctr);
-        CKL();
-    }
-    CK(cudaMemcpyAsync(&G->ctr_host->status, &G->ctr->status, sizeof(unsigned),
-                       cudaMemcpyDeviceToHost, G->stream));
-    CK(cudaMemcpyAsync(G->hx, &G->ctr->pool_cursor, sizeof(int64_t), cudaMemcpyDeviceToHost,
-                       G->stream));
-    CK(cudaStreamSynchronize(G->stream));
-    if (G->ctr_host->status) {
-        CK(cudaMemsetAsync(&G->ctr->status, 0, sizeof(unsigned), G->stream));
-        CK(cudaMemsetAsync(G->deg, 0, sizeof(int32_t) * (size_t)(n_after + 1), G->stream));
-        return fail(G, PIRRT_ERR_BAD_INPUT,
-                    "insert_batch: edge with an id outside [0, %lld), a self loop, or a cost "
-                    "that is not finite and > 0",
-                    (long long)n_after);
-    }
-    const int64_t need = G->hx[0];
-    // 3. move those rows to the end of the pool, or repack every row into the
-    //    other pool when this one is used up; set every changed row's new length
-    if (G->pool_used + need <= G->pool_cap) {
-        if (changed_max > 0) {
-            Entry<CT> *pool = static_cast<Entry<CT> *>(G->adj[G->cur]);
-            insert_move_list<CT><<<grid_for((changed_max + 31) / 32 * 32, kThreads, max_blocks),
-                                   kThreads, 0, G->stream>>>(
-                n_old, n_after, G->touched, G->rows, G->deg, G->ralloc, G->roff,
-                (long long)G->pool_used, pool, G->ctr);
+    InsertReport *rep = G->insert_rep;
+    if (n_edges > 0 || n_new > 0) {
+        InsertArgs<CT> a{};
+        a.n_edges = n_edges;
+        a.n_old = n_old;
+        a.n_after = n_after;
+        a.src = src;
+        a.dst = dst;
+        a.cost = cost;
+        a.root = G->cfg.root;
+        a.seq = ++G->insert_seq;
+        a.rows = G->rows;
+        a.deg = G->deg;
+        a.touched = G->touched;
+        a.alloc = G->ralloc;
+        a.off = G->roff;
+        a.pool = static_cast<Entry<CT> *>(G->adj[G->cur]);
+        a.pool_used = (long long)G->pool_used;
+        a.pool_cap = (long long)G->pool_cap;
+        a.g = G->g;
+        a.g32 = G->g32;
+        a.p = G->p;
+        a.pc = static_cast<CT *>(G->pc);
+        a.cand = G->cand;
+        a.stamp = G->stamp;
+        a.list[0] = G->list[0];
+        a.list[1] = G->list[1];
+        a.ctr = G->ctr;
+        a.report = rep;
+        // no more CTAs than the block keeps busy: a barrier costs its arrivals
+        const int64_t items = std::max<int64_t>((n_edges + kInsertUnroll - 1) / kInsertUnroll, n_new);
+        const int blocks = grid_for(items, kInsertThreads, G->insert_blocks);
+        void *args[] = {&a};
+        CK(cudaLaunchCooperativeKernel((const void *)insert_kernel<CT>, dim3(blocks),
+                                       dim3(kInsertThreads), args, 0, G->stream));
+        // the report comes before the entries are written
+        for (unsigned polls = 0; *const_cast<volatile unsigned *>(&rep->seq) != a.seq; ++polls) {
+            if ((polls & 1023u) != 1023u) continue;
+            const cudaError_t e = cudaStreamQuery(G->stream);
+            if (e == cudaErrorNotReady) continue;
+            CK(e);
+            if (*const_cast<volatile unsigned *>(&rep->seq) != a.seq)
+                return fail(G, PIRRT_ERR_CUDA, "insert_batch: the kernel left no report");
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
+        G->prof.launches += 1;
+        if (rep->status || rep->late) {
+            insert_clear_kernel<<<1, 1, 0, G->stream>>>(G->ctr);
             CKL();
-        }
-        G->pool_used += need;
-    } else {
-        const int move_blocks = grid_for((n_after + 31) / 32 * 32, kThreads, max_blocks);
-        const int nxt = G->cur ^ 1;
-        if (!G->adj[nxt]) {
-            const cudaError_t e =
-                cudaMalloc(&G->adj[nxt], G->entry_bytes * (size_t)(G->pool_cap + 16));
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                G->adj[nxt] = nullptr;
-                CK(cudaMemsetAsync(G->deg, 0, sizeof(int32_t) * (size_t)(n_after + 1), G->stream));
-                return fail(G, PIRRT_ERR_OOM, "insert_batch: no memory for a second CSR pool");
-            }
-        }
-        if (const pirrt_status rc = insert_plan_scan(G, n_old, n_after, 1)) return rc;
-        CK(cudaMemcpyAsync(G->hx, &G->roff[n_after], sizeof(int64_t), cudaMemcpyDeviceToHost,
-                           G->stream));
-        CK(cudaStreamSynchronize(G->stream));
-        const int64_t total = G->hx[0];
-        if (total > G->pool_cap) {
             CK(cudaMemsetAsync(G->deg, 0, sizeof(int32_t) * (size_t)(n_after + 1), G->stream));
-            return fail(G, PIRRT_ERR_CAPACITY, "insert_batch: repacked CSR needs %lld entries",
-                        (long long)total);
+            if (!(rep->status & kStatusBadInput))
+                return fail(G, PIRRT_ERR_DEVICE_TIMEOUT, "insert_batch: a grid barrier timed out");
+            return fail(G, PIRRT_ERR_BAD_INPUT,
+                        "insert_batch: edge with an id outside [0, %lld), a self loop, or a cost "
+                        "that is not finite and > 0",
+                        (long long)n_after);
         }
-        insert_move_rows<CT><<<move_blocks, kThreads, 0, G->stream>>>(
-            n_old, n_after, G->rows, G->deg, G->ralloc, G->roff, 0ll,
-            static_cast<const Entry<CT> *>(G->adj[G->cur]), static_cast<Entry<CT> *>(G->adj[nxt]),
-            G->ctr, 1);
-        CKL();
-        G->cur = nxt;
-        G->pool_used = total;
-        G->prof.launches += 4;
+        const int64_t need = (int64_t)rep->need;
+        if (G->pool_used + need <= G->pool_cap) {
+            G->pool_used += need;
+        } else {
+            // the kernel has stopped there: repack every row into the other
+            // pool, then run the last passes
+            insert_clear_kernel<<<1, 1, 0, G->stream>>>(G->ctr);
+            CKL();
+            const int max_blocks = G->num_sms * 32;
+            const int move_blocks = grid_for((n_after + 31) / 32 * 32, kThreads, max_blocks);
+            const int nxt = G->cur ^ 1;
+            if (!G->adj[nxt]) {
+                const cudaError_t e =
+                    cudaMalloc(&G->adj[nxt], G->entry_bytes * (size_t)(G->pool_cap + 16));
+                if (e != cudaSuccess) {
+                    cudaGetLastError();
+                    G->adj[nxt] = nullptr;
+                    CK(cudaMemsetAsync(G->deg, 0, sizeof(int32_t) * (size_t)(n_after + 1), G->stream));
+                    return fail(G, PIRRT_ERR_OOM, "insert_batch: no memory for a second CSR pool");
+                }
+            }
+            if (const pirrt_status rc = insert_plan_scan(G, n_old, n_after, 1)) return rc;
+            CK(cudaMemcpyAsync(G->hx, &G->roff[n_after], sizeof(int64_t), cudaMemcpyDeviceToHost,
+                               G->stream));
+            CK(cudaStreamSynchronize(G->stream));
+            const int64_t total = G->hx[0];
+            if (total > G->pool_cap) {
+                CK(cudaMemsetAsync(G->deg, 0, sizeof(int32_t) * (size_t)(n_after + 1), G->stream));
+                return fail(G, PIRRT_ERR_CAPACITY, "insert_batch: repacked CSR needs %lld entries",
+                            (long long)total);
+            }
+            insert_move_rows<CT><<<move_blocks, kThreads, 0, G->stream>>>(
+                n_old, n_after, G->rows, G->deg, G->ralloc, G->roff, 0ll,
+                static_cast<const Entry<CT> *>(G->adj[G->cur]),
+                static_cast<Entry<CT> *>(G->adj[nxt]), G->ctr, 1);
+            CKL();
+            G->cur = nxt;
+            G->pool_used = total;
+            a.pool = static_cast<Entry<CT> *>(G->adj[nxt]);
+            // seed before the entries, whose offers may reach the new vertices
+            if (n_new > 0) {
+                insert_init_kernel<CT><<<grid_for(n_new, kInsertThreads, G->insert_blocks),
+                                         kInsertThreads, 0, G->stream>>>(a);
+                CKL();
+            }
+            if (n_edges > 0) {
+                insert_entries_kernel<CT><<<blocks, kInsertThreads, 0, G->stream>>>(a);
+                CKL();
+            }
+            G->prof.launches += 6 + (n_new > 0) + (n_edges > 0);
+        }
     }
-    Entry<CT> *new_adj = static_cast<Entry<CT> *>(G->adj[G->cur]);
-    // 4. seed the new vertices (before the scatter, whose offers may reach them)
-    if (n_new > 0) {
-        insert_init_vertices<CT><<<grid_for(n_new, kThreads, max_blocks), kThreads, 0, G->stream>>>(
-            n_old, n_after, G->cfg.root, G->g, G->g32, G->p, static_cast<CT *>(G->pc), G->cand,
-            G->stamp, G->list[0], G->list[1], G->ctr);
-        CKL();
-    }
-    // 5. new entries at the row tails
-    if (n_edges > 0) {
-        insert_scatter<CT><<<grid_for(n_edges, kThreads, max_blocks), kThreads, 0, G->stream>>>(
-            n_edges, src, dst, cost, G->rows, G->deg, new_adj, G->stamp, G->cfg.root,
-            G->list[0], G->list[1], G->g, G->cand, G->ctr);
-        CKL();
-    }
-    G->prof.launches += 1 + (n_edges > 0 ? 2 : 0) + (changed_max > 0 ? 2 : 0) + (n_new > 0 ? 1 : 0);
     G->prof.insert_calls += 1;
     G->prof.insert_new_entries += 2 * n_edges;
     if (prof) {
@@ -1162,6 +1182,7 @@ void free_all(pirrt_graph *G) {
         if (q) cudaFree(q);
     if (G->ctr_host) cudaFreeHost(G->ctr_host);
     if (G->hx) cudaFreeHost(G->hx);
+    if (G->insert_rep) cudaFreeHost(G->insert_rep);
     if (G->loop_res) cudaFreeHost(G->loop_res);
     if (G->ev0) cudaEventDestroy(G->ev0);
     if (G->ev1) cudaEventDestroy(G->ev1);
@@ -1377,6 +1398,9 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
         return bail(PIRRT_ERR_CUDA);
     if (cudaMallocHost((void **)&G->hx, 2 * sizeof(int64_t)) != cudaSuccess)
         return bail(PIRRT_ERR_OOM);
+    if (cudaMallocHost((void **)&G->insert_rep, sizeof(InsertReport)) != cudaSuccess)
+        return bail(PIRRT_ERR_OOM);
+    *G->insert_rep = InsertReport{};
     if (cudaMallocHost((void **)&G->ctr_host, sizeof(DevCounters)) != cudaSuccess)
         return bail(PIRRT_ERR_OOM);
     if (cudaMallocHost((void **)&G->loop_res, sizeof(LoopResult)) != cudaSuccess)
@@ -1423,6 +1447,15 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     locc = std::min(locc, locc64);
     if (locc < 1) return bail(PIRRT_ERR_CUDA);
     G->loop_occ = std::min(locc, 2);
+    int iocc = 0, iocc64 = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&iocc, insert_kernel<float>, kInsertThreads,
+                                                      0) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&iocc64, insert_kernel<double>, kInsertThreads,
+                                                      0) != cudaSuccess)
+        return bail(PIRRT_ERR_CUDA);
+    iocc = std::min(iocc, iocc64);
+    if (iocc < 1) return bail(PIRRT_ERR_CUDA);
+    G->insert_blocks = G->num_sms * std::min(iocc, 3);
     int aocc = 0, aocc64 = 0;
     if (cudaFuncSetAttribute(async_evaluate_kernel<float>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAsyncSmem) !=
@@ -1466,6 +1499,7 @@ pirrt_status pirrt_graph_reset(pirrt_graph *G) {
     CK(cudaMemcpyAsync(&G->ctr->wave_epoch, &one, sizeof(unsigned), cudaMemcpyHostToDevice,
                        G->stream));
     CK(cudaStreamSynchronize(G->stream));
+    *G->insert_rep = InsertReport{};
     G->pool_used = 0;
     G->copied_seen = 0;
     G->n = 0;
@@ -1637,6 +1671,8 @@ pirrt_status pirrt_graph_exploit(pirrt_graph *G, const pirrt_exploit_opts *opts,
     const pirrt_status rc = G->cfg.cost_dtype == PIRRT_COST_F32 ? exploit_impl<float>(G, opts, stats)
                                                                 : exploit_impl<double>(G, opts, stats);
     if (rc != PIRRT_OK) G->async_dirty = 1;
+    if (rc == PIRRT_OK && *const_cast<volatile unsigned *>(&G->insert_rep->late))
+        return fail(G, PIRRT_ERR_DEVICE_TIMEOUT, "insert_batch: a grid barrier timed out");
     return rc;
 }
 
