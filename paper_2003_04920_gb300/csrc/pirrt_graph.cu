@@ -809,11 +809,19 @@ pirrt_status exploit_loop(pirrt_graph *G, const pirrt_exploit_opts &o, bool jump
     a.local_step = o.wave_local_step > 0 ? (unsigned)o.wave_local_step : 512u;
     const int occ = o.wave_ctas > 0 ? std::min(o.wave_ctas, G->loop_occ) : G->loop_occ;
     int blocks = G->num_sms * occ;
-    blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(8, (G->n + 127) / 128));
+    // a policy that fits shared memory is walked there, with the CTAs that leaves
+    // every one its share of the vertices (loop_walk)
+    constexpr int per = sizeof(CT) == 4 ? kWalkPer : kWalkPerF64;
+    constexpr int64_t most = sizeof(CT) == 4 ? kWalkVertices : kWalkVerticesF64;
+    a.walk = G->n <= std::min<int64_t>(most, (int64_t)per * G->num_sms) ? 1 : 0;
+    const int64_t share = a.walk ? per : 128;
+    blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(8, (G->n + share - 1) / share));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(kLoopThreads);
     cfg.dynamicSmemBytes = sizeof(LoopShared<CT>);
+    if (a.walk)
+        cfg.dynamicSmemBytes = ((cfg.dynamicSmemBytes + 15) & ~size_t(15)) + walk_bytes<CT>(G->n);
     cfg.stream = G->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -1434,10 +1442,13 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     G->wave_occ = std::min(wocc, 2);
     G->wave_blocks = G->num_sms * G->wave_occ;
     int locc = 0, locc64 = 0;
-    if (cudaFuncSetAttribute(replan_loop_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(LoopShared<float>)) != cudaSuccess ||
-        cudaFuncSetAttribute(replan_loop_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(LoopShared<double>)) != cudaSuccess ||
+    if (cudaFuncSetAttribute(
+            replan_loop_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            (int)(sizeof(LoopShared<float>) + 16 + walk_bytes<float>(kWalkVertices))) != cudaSuccess ||
+        cudaFuncSetAttribute(
+            replan_loop_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            (int)(sizeof(LoopShared<double>) + 16 + walk_bytes<double>(kWalkVerticesF64))) !=
+            cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&locc, replan_loop_kernel<float>, kLoopThreads,
                                                       sizeof(LoopShared<float>)) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&locc64, replan_loop_kernel<double>,

@@ -86,6 +86,7 @@ struct LoopArgs {
     int32_t jump;         // every Evaluate by pointer jumping
     int32_t hops;         // links followed per pointer-jumping round
     int32_t top_rounds;   // FP64 costs: rounds summed from the root down before it
+    int32_t walk;         // the policy fits shared memory: each vertex walks up to the root
     unsigned max_iters;
     unsigned dense_limit, max_levels;
     unsigned tail_max, local_levels, local_max, local_step;
@@ -1012,6 +1013,142 @@ __device__ __forceinline__ bool loop_jump(const LoopArgs<CT> &a, LoopCounters *i
     return true;
 }
 
+// The same for a policy that fits shared memory: every CTA loads all of it
+// (coalesced, out of L2) and walks up from its own vertices, a link being a
+// shared-memory round trip (some 30 cycles) instead of an L2 one (302), to the
+// root in one go: no records, no rounds, one barrier.  With FP32 costs a vertex's
+// sum runs from itself upwards, as in loop_jump; with FP64 costs, whose sums
+// round, the links are kept on a stack and added from the root down, as Alg. 2
+// adds them, up to the depth that top_round covers.  A vertex deeper than that, or
+// below a cycle, sends the whole Evaluate to loop_jump, which finds the others
+// as it would leave them (and the rest of the exploit goes there at once).
+// At most 128 vertices a CTA (64 with stacks): with one warp per scheduler the
+// slow FP64 additions hide behind the loads.
+//
+// Measured, ms of exploit by loop_jump and by loop_walk: 10,000 vertices in 2-D in
+// 100 goal-directed blocks 16.7 and 15.2, 3,000 in 20 blocks 3.52 and 2.81, 10,000
+// in 6-D in 10 blocks 1.48 and 1.22; a policy of 2,000 with FP64 costs 0.241 and
+// 0.145, of 9,500 0.65 and 0.32; FP64 blocks up to 9,700 in 2-D 6.9 and 3.6.  The
+// limits are what shared memory holds beside the loop's own; at 16,000 vertices
+// 0.434 and 0.408, at 19,000 (where the L1 cache left over shrinks further) 0.416
+// and 0.445.
+constexpr int64_t kWalkVertices = 16384, kWalkVerticesF64 = 9728;
+constexpr int kWalkPer = 128;    // vertices of a CTA: one warp per scheduler
+constexpr int kWalkPerF64 = 64;  // ... FP64 costs, whose stacks take room
+constexpr int kWalkDepth = 96;   // FP64 costs: links kept to be added from the root down
+
+// Shared memory beyond LoopShared.
+template <typename CT>
+constexpr size_t walk_bytes(int64_t n) {
+    return sizeof(CT) == 4 ? 8 * (size_t)((n + 3) & ~3ll)
+                           : 12 * (size_t)((n + 3) & ~3ll) + 8 * (size_t)(kWalkDepth * kWalkPerF64);
+}
+
+template <typename CT>
+__device__ __forceinline__ bool loop_walk(const LoopArgs<CT> &a, LoopCounters *ic, bool stale,
+                                          bool &walk) {
+    LoopShared<CT> &sh = loop_shared<CT>();
+    constexpr size_t kAt = (sizeof(LoopShared<CT>) + 15) & ~size_t(15);
+    unsigned char *mem = reinterpret_cast<unsigned char *>(&sh) + kAt;
+    const int n = (int)a.n, n4 = n & ~3;
+    const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int v = (int)blockIdx.x * per + (int)threadIdx.x;
+    bool open = false, changed = false;
+    unsigned finished = 0;
+    // the whole policy, 16 bytes a load
+    int2 *link = reinterpret_cast<int2 *>(mem);                 // FP32: {parent, cost}
+    double *cost = reinterpret_cast<double *>(mem);             // FP64: costs, parents, stack
+    int32_t *par = reinterpret_cast<int32_t *>(mem + 8 * (size_t)((n + 3) & ~3));
+    double *stack = reinterpret_cast<double *>(mem + 12 * (size_t)((n + 3) & ~3));
+    for (int i = 4 * (int)threadIdx.x; i < n4; i += 4 * kLoopThreads) {
+        const int4 q = __ldcg(reinterpret_cast<const int4 *>(a.p + i));
+        if constexpr (sizeof(CT) == 4) {
+            const int4 w = __ldcg(reinterpret_cast<const int4 *>(a.pc + i));
+            *reinterpret_cast<int4 *>(link + i) = make_int4(q.x, w.x, q.y, w.y);
+            *reinterpret_cast<int4 *>(link + i + 2) = make_int4(q.z, w.z, q.w, w.w);
+        } else {
+            *reinterpret_cast<int4 *>(par + i) = q;
+            const int4 *w = reinterpret_cast<const int4 *>(a.pc + i);
+            reinterpret_cast<int4 *>(cost + i)[0] = __ldcg(w);
+            reinterpret_cast<int4 *>(cost + i)[1] = __ldcg(w + 1);
+        }
+    }
+    for (int i = n4 + (int)threadIdx.x; i < n; i += kLoopThreads) {
+        if constexpr (sizeof(CT) == 4) {
+            link[i] = make_int2(__ldcg(a.p + i), __float_as_int(__ldcg(a.pc + i)));
+        } else {
+            par[i] = __ldcg(a.p + i);
+            cost[i] = __ldcg(a.pc + i);
+        }
+    }
+    double old = 0.0;
+    const bool mine = (int)threadIdx.x < per && v < n;
+    if (mine) old = __ldcg(&a.g[v]);
+    __syncthreads();
+    if (mine) {
+        double gw = 0.0;
+        bool has = false;
+        if constexpr (sizeof(CT) == 4) {
+            int2 t = link[v];
+            if (t.x >= 0) {
+                has = true;
+                double s = (double)__int_as_float(t.y);
+                int x = t.x, hops = 0;
+                for (t = link[x]; t.x >= 0; t = link[x]) {
+                    s += (double)__int_as_float(t.y);
+                    x = t.x;
+                    if (++hops > n) {  // a cycle: left to pointer jumping, which reports it
+                        open = true;
+                        break;
+                    }
+                }
+                gw = s + __ldcg(&a.g[x]);
+            }
+        } else {
+            int x = par[v];
+            if (x >= 0) {
+                has = true;
+                stack[threadIdx.x] = cost[v];
+                int d = 1;
+                for (int up = par[x]; up >= 0; up = par[x]) {
+                    if (d == kWalkDepth) {
+                        open = true;
+                        break;
+                    }
+                    stack[d++ * kWalkPerF64 + threadIdx.x] = cost[x];
+                    x = up;
+                }
+                gw = __ldcg(&a.g[x]);
+                while (--d >= 0) gw = gw + stack[d * kWalkPerF64 + threadIdx.x];
+            }
+        }
+        if (has && !open) {
+            const bool diff = __double_as_longlong(gw) != __double_as_longlong(old);
+            if (diff) a.g[v] = gw;
+            // a wave leaves the FP32 shadow behind: every one is rewritten then
+            if (diff || stale) a.g32[v] = g32_of(gw);
+            changed = diff;
+            finished = 1u;
+        }
+    }
+    if (changed) sh.mark[atomicAdd(&sh.nmark, 1u)] = v;
+    const unsigned left = __syncthreads_or(open) ? 1u : 0u;
+    flush_marks<CT>(sh, a.dg, &ic->n_jump);
+    if (!loop_sync<CT>(a.ctr, sh, left)) return false;
+    if (sh.total != 0u) {
+        walk = false;
+        return loop_jump<CT>(a, ic, stale);
+    }
+    if (threadIdx.x == 0) {
+        sh.rounds = 1u;
+        sh.bad = 0u;
+    }
+    add_total(finished, &sh.tot[2]);
+    __syncthreads();
+    return true;
+}
+
+
 // After pointer jumping: every changed vertex offers its neighbours their
 // candidate through it where it beats their g, and lists them.  L lanes per
 // changed vertex.
@@ -1148,6 +1285,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
     unsigned iter = 0, levels_sum = 0, dense_sum = 0, rounds_sum = 0, jump_sum = 0;
     unsigned long long switches = 0;  // thread 0
     bool converged = false, ok = true;
+    bool walk = a.walk != 0;  // ... until a policy is too deep for it
     LoopCounters *ic = &c->loop[par];
     __syncthreads();
     if (sizeof(CT) == 4 && dense && stale) {
@@ -1248,7 +1386,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
             if (jump) {
                 // ---- Evaluate, or the rest of a wave too deep, by pointer jumping
                 const long long tj = clock64();
-                ok = loop_jump<CT>(a, ic, stale);
+                ok = walk ? loop_walk<CT>(a, ic, stale, walk) : loop_jump<CT>(a, ic, stale);
                 if (tid == 0 && sh.tr.state != -1)
                     c->ph_jump_cyc += (unsigned long long)(clock64() - tj);
                 if (!ok) break;
