@@ -146,6 +146,8 @@ struct DevCounters {
     alignas(128) unsigned wl_count[kMaxJumpRounds + 2];  // pointer-jumping work-list sizes per round
     alignas(128) unsigned n_touched;   // insertion: old rows gaining entries (list length)
     unsigned insert_status;            // ... kStatus* bits
+    alignas(128) unsigned sig_ticket;  // signal_host: CTAs done
+    unsigned sig_status;               // ... kStatus* bits to tell the host
     alignas(128) unsigned long long pool_cursor;  // insertion: pool room taken by the block
     alignas(128) unsigned status;      // kStatus* bits
     unsigned long long switches;  // parent switches (whole exploit)
@@ -201,6 +203,31 @@ struct DevCounters {
     unsigned long long t_enter, t_last_exit, span_ns, spans, gap_ns, gaps;
     unsigned long long ph_pre_cyc, ph_post_cyc, ph_jump_cyc, ph_calls;
 };
+
+// What a short kernel tells the host when its work is done, in page-locked
+// memory; seq is written last.  The host polls it: for calls of a few
+// microseconds the copy of a status word and the wake-up after the stream's end
+// (8 us and more) are most of the time.
+struct HostSignal {
+    unsigned status;  // kStatus* bits
+    unsigned seq;     // number of the call
+};
+
+// End of a kernel of any grid: the last CTA to get here reports.  Every thread of
+// the CTA calls it.
+__device__ __forceinline__ void signal_host(DevCounters *c, HostSignal *host, unsigned seq) {
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(&c->sig_ticket, 1u) != gridDim.x - 1u) return;
+    __threadfence();
+    volatile HostSignal *h = host;
+    h->status = __ldcg(&c->sig_status);
+    c->sig_ticket = 0u;
+    c->sig_status = 0u;
+    __threadfence_system();
+    h->seq = seq;
+}
 
 // Block-wide sum of one value per thread, added to *counter by one atomic.
 // Every thread of the block must call it; s needs blockDim.x / 32 entries.

@@ -1204,10 +1204,21 @@ static __global__ void refresh_g32_done(DevCounters *c, int always_if_stale) {
 
 // Parents as reported through the ABI: the root marker becomes -1.
 static __global__ void export_parents_kernel(int64_t n, const int32_t *__restrict__ p,
-                                             int32_t *__restrict__ out) {
+                                             int32_t *__restrict__ out, DevCounters *c,
+                                             HostSignal *host, unsigned seq) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x)
         out[v] = p[v] < 0 ? -1 : p[v];
+    signal_host(c, host, seq);
+}
+
+static __global__ void export_costs_kernel(int64_t n, const double *__restrict__ g,
+                                           double *__restrict__ out, DevCounters *c,
+                                           HostSignal *host, unsigned seq) {
+    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
+         v += (int64_t)gridDim.x * blockDim.x)
+        out[v] = g[v];
+    signal_host(c, host, seq);
 }
 
 // Batched form: translate one graph's local edge ids into the union graph
@@ -1218,12 +1229,13 @@ __global__ void __launch_bounds__(kThreads)
 batch_translate_kernel(int64_t n_edges, const int32_t *__restrict__ src,
                        const int32_t *__restrict__ dst, const CT *__restrict__ cost, int64_t base,
                        int64_t limit, int32_t *__restrict__ out_src, int32_t *__restrict__ out_dst,
-                       CT *__restrict__ out_cost, DevCounters *ctr) {
+                       CT *__restrict__ out_cost, DevCounters *ctr, HostSignal *host,
+                       unsigned seq) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n_edges;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int32_t a = src[e], b = dst[e];
         if (a < 0 || b < 0 || a >= limit || b >= limit) {
-            atomicOr(&ctr->status, kStatusBadInput);
+            atomicOr(&ctr->sig_status, kStatusBadInput);
             out_src[e] = 0;
             out_dst[e] = 0;  // rejected by the union validation as a self loop
             out_cost[e] = CT(0);
@@ -1233,17 +1245,20 @@ batch_translate_kernel(int64_t n_edges, const int32_t *__restrict__ src,
         out_dst[e] = (int32_t)(b + base);
         out_cost[e] = cost[e];
     }
+    signal_host(ctr, host, seq);
 }
 
 // Batched form: parents of one graph in its own ids (root marker -> -1).
 static __global__ void export_parents_local_kernel(int64_t n, int64_t base,
                                                    const int32_t *__restrict__ p,
-                                                   int32_t *__restrict__ out) {
+                                                   int32_t *__restrict__ out, DevCounters *c,
+                                                   HostSignal *host, unsigned seq) {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int32_t q = p[base + v];
         out[v] = q < 0 ? -1 : (int32_t)(q - base);
     }
+    signal_host(c, host, seq);
 }
 
 // Make each listed vertex a root: g = 0, parent marker kRootMark.

@@ -67,6 +67,8 @@ struct pirrt_graph {
     int64_t *hx = nullptr;         // pinned host scalars read back by insertion
     InsertReport *insert_rep = nullptr;  // pinned: what an insertion's kernel tells the host
     unsigned insert_seq = 0;
+    HostSignal *sig = nullptr;           // pinned: the end of a read-back, or of a batch insert
+    unsigned sig_seq = 0;
     int insert_blocks = 0;               // co-resident grid of the insertion kernel
     double *g = nullptr;
     float *g32 = nullptr;  // FP32 shadow of g for candidate screening
@@ -178,6 +180,58 @@ pirrt_status status_from_bits(pirrt_graph *G, unsigned bits) {
 // Read the counter block back (synchronises the stream).
 pirrt_status pull_counters(pirrt_graph *G) {
     CK(cudaMemcpyAsync(G->ctr_host, G->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, G->stream));
+    CK(cudaStreamSynchronize(G->stream));
+    return PIRRT_OK;
+}
+
+// Poll a word in page-locked memory that a kernel of the graph's stream sets to
+// `seq`.  The stream itself is asked now and then, so that a failed kernel ends
+// the wait.
+pirrt_status wait_host(pirrt_graph *G, const unsigned *word, unsigned seq) {
+    const volatile unsigned *w = word;
+    for (unsigned polls = 0; *w != seq; ++polls) {
+        if ((polls & 1023u) != 1023u) continue;
+        const cudaError_t e = cudaStreamQuery(G->stream);
+        if (e == cudaErrorNotReady) continue;
+        CK(e);
+        if (*w != seq) return fail(G, PIRRT_ERR_CUDA, "a kernel left no report");
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return PIRRT_OK;
+}
+
+// Device memory of the graph's own GPU, which its kernels can write (a copy
+// reaches any other).
+bool own_memory(const pirrt_graph *G, const void *p) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == G->cfg.device;
+}
+
+// n costs from `from` into the caller's buffer, complete on return.
+pirrt_status costs_out(pirrt_graph *G, const double *from, double *out, int64_t n, int on_device) {
+    if (n > 0 && on_device && own_memory(G, out)) {
+        export_costs_kernel<<<grid_for(n, kThreads, G->num_sms * 8), kThreads, 0, G->stream>>>(
+            n, from, out, G->ctr, G->sig, ++G->sig_seq);
+        CKL();
+        return wait_host(G, &G->sig->seq, G->sig_seq);
+    }
+    if (n > 0)
+        CK(cudaMemcpyAsync(out, from, sizeof(double) * (size_t)n,
+                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, G->stream));
+    CK(cudaStreamSynchronize(G->stream));
+    return PIRRT_OK;
+}
+
+// The end of a parents read-back whose kernel (number sig_seq) has been launched:
+// straight into the caller's device buffer, or through pexport to the host.
+pirrt_status parents_out(pirrt_graph *G, int32_t *out, int64_t n, int on_device) {
+    if (on_device) return wait_host(G, &G->sig->seq, G->sig_seq);
+    CK(cudaMemcpyAsync(out, G->pexport, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost,
+                       G->stream));
     CK(cudaStreamSynchronize(G->stream));
     return PIRRT_OK;
 }
@@ -665,15 +719,7 @@ pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const i
         CK(cudaLaunchCooperativeKernel((const void *)insert_kernel<CT>, dim3(blocks),
                                        dim3(kInsertThreads), args, 0, G->stream));
         // the report comes before the entries are written
-        for (unsigned polls = 0; *const_cast<volatile unsigned *>(&rep->seq) != a.seq; ++polls) {
-            if ((polls & 1023u) != 1023u) continue;
-            const cudaError_t e = cudaStreamQuery(G->stream);
-            if (e == cudaErrorNotReady) continue;
-            CK(e);
-            if (*const_cast<volatile unsigned *>(&rep->seq) != a.seq)
-                return fail(G, PIRRT_ERR_CUDA, "insert_batch: the kernel left no report");
-        }
-        std::atomic_thread_fence(std::memory_order_acquire);
+        if (const pirrt_status rc = wait_host(G, &rep->seq, a.seq)) return rc;
         G->prof.launches += 1;
         if (rep->status || rep->late) {
             insert_clear_kernel<<<1, 1, 0, G->stream>>>(G->ctr);
@@ -1191,6 +1237,7 @@ void free_all(pirrt_graph *G) {
     if (G->ctr_host) cudaFreeHost(G->ctr_host);
     if (G->hx) cudaFreeHost(G->hx);
     if (G->insert_rep) cudaFreeHost(G->insert_rep);
+    if (G->sig) cudaFreeHost(G->sig);
     if (G->loop_res) cudaFreeHost(G->loop_res);
     if (G->ev0) cudaEventDestroy(G->ev0);
     if (G->ev1) cudaEventDestroy(G->ev1);
@@ -1264,17 +1311,14 @@ template <typename CT>
 pirrt_status batch_translate(pirrt_batch *B, int32_t graph, int64_t n_edges, const int32_t *src,
                              const int32_t *dst, const CT *cost) {
     pirrt_graph *G = B->G;
-    CK(cudaMemsetAsync(&G->ctr->status, 0, sizeof(unsigned), G->stream));
     batch_translate_kernel<CT><<<grid_for(n_edges, kThreads, G->num_sms * 32), kThreads, 0,
                                  G->stream>>>(
         n_edges, src, dst, cost, B->base[graph], B->cap_v[graph], B->pend_src + B->pend_n,
-        B->pend_dst + B->pend_n, static_cast<CT *>(B->pend_cost) + B->pend_n, G->ctr);
+        B->pend_dst + B->pend_n, static_cast<CT *>(B->pend_cost) + B->pend_n, G->ctr, G->sig,
+        ++G->sig_seq);
     CKL();
-    CK(cudaMemcpyAsync(&G->ctr_host->status, &G->ctr->status, sizeof(unsigned),
-                       cudaMemcpyDeviceToHost, G->stream));
-    CK(cudaStreamSynchronize(G->stream));
-    if (G->ctr_host->status) {
-        CK(cudaMemsetAsync(&G->ctr->status, 0, sizeof(unsigned), G->stream));
+    if (const pirrt_status rc = wait_host(G, &G->sig->seq, G->sig_seq)) return rc;
+    if (G->sig->status) {
         return fail(G, PIRRT_ERR_BAD_INPUT, "batch_insert: an id outside [0, %lld) of graph %d",
                     (long long)B->cap_v[graph], graph);
     }
@@ -1409,6 +1453,9 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     if (cudaMallocHost((void **)&G->insert_rep, sizeof(InsertReport)) != cudaSuccess)
         return bail(PIRRT_ERR_OOM);
     *G->insert_rep = InsertReport{};
+    if (cudaMallocHost((void **)&G->sig, sizeof(HostSignal)) != cudaSuccess)
+        return bail(PIRRT_ERR_OOM);
+    *G->sig = HostSignal{};
     if (cudaMallocHost((void **)&G->ctr_host, sizeof(DevCounters)) != cudaSuccess)
         return bail(PIRRT_ERR_OOM);
     if (cudaMallocHost((void **)&G->loop_res, sizeof(LoopResult)) != cudaSuccess)
@@ -1694,11 +1741,7 @@ pirrt_status pirrt_graph_get_costs(const pirrt_graph *Gc, double *g_out, int64_t
         return fail(G, PIRRT_ERR_INVALID_ARG, "get_costs: n = %lld but the graph has %lld vertices",
                     (long long)n, (long long)G->n);
     CK(cudaSetDevice(G->cfg.device));
-    if (n > 0)
-        CK(cudaMemcpyAsync(g_out, G->g, sizeof(double) * (size_t)n,
-                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, G->stream));
-    CK(cudaStreamSynchronize(G->stream));
-    return PIRRT_OK;
+    return costs_out(G, G->g, g_out, n, on_device);
 }
 
 pirrt_status pirrt_graph_get_parents(const pirrt_graph *Gc, int32_t *p_out, int64_t n, int on_device) {
@@ -1711,11 +1754,9 @@ pirrt_status pirrt_graph_get_parents(const pirrt_graph *Gc, int32_t *p_out, int6
     if (n > 0) {
         int32_t *dst = on_device ? p_out : G->pexport;
         export_parents_kernel<<<grid_for(n, kThreads, G->num_sms * 8), kThreads, 0, G->stream>>>(
-            n, G->p, dst);
+            n, G->p, dst, G->ctr, G->sig, ++G->sig_seq);
         CKL();
-        if (!on_device)
-            CK(cudaMemcpyAsync(p_out, G->pexport, sizeof(int32_t) * (size_t)n,
-                               cudaMemcpyDeviceToHost, G->stream));
+        return parents_out(G, p_out, n, on_device);
     }
     CK(cudaStreamSynchronize(G->stream));
     return PIRRT_OK;
@@ -2322,11 +2363,7 @@ pirrt_status pirrt_batch_get_costs(const pirrt_batch *B, int32_t graph, double *
         return PIRRT_ERR_INVALID_ARG;
     pirrt_graph *G = B->G;
     CK(cudaSetDevice(G->cfg.device));
-    if (n > 0)
-        CK(cudaMemcpyAsync(g_out, G->g + B->base[graph], sizeof(double) * (size_t)n,
-                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, G->stream));
-    CK(cudaStreamSynchronize(G->stream));
-    return PIRRT_OK;
+    return costs_out(G, G->g + B->base[graph], g_out, n, on_device);
 }
 
 pirrt_status pirrt_batch_get_parents(const pirrt_batch *B, int32_t graph, int32_t *p_out, int64_t n,
@@ -2338,11 +2375,10 @@ pirrt_status pirrt_batch_get_parents(const pirrt_batch *B, int32_t graph, int32_
     if (n > 0) {
         int32_t *dst = on_device ? p_out : G->pexport;
         export_parents_local_kernel<<<grid_for(n, kThreads, G->num_sms * 8), kThreads, 0,
-                                      G->stream>>>(n, B->base[graph], G->p, dst);
+                                      G->stream>>>(n, B->base[graph], G->p, dst, G->ctr, G->sig,
+                                                   ++G->sig_seq);
         CKL();
-        if (!on_device)
-            CK(cudaMemcpyAsync(p_out, G->pexport, sizeof(int32_t) * (size_t)n,
-                               cudaMemcpyDeviceToHost, G->stream));
+        return parents_out(G, p_out, n, on_device);
     }
     CK(cudaStreamSynchronize(G->stream));
     return PIRRT_OK;
