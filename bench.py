@@ -309,7 +309,7 @@ def run_ours(args) -> None:
 
     # device-resident inputs, one CUDA-event pair per step, L2 flushed between
     # steps outside the timed spans (the CSR is also ~8x larger than L2).
-    # "graph": every exploit is one CUDA-graph launch (the product path), and
+    # "graph": every exploit is one launch (the product path), and
     # the per-kernel split comes from profiled steps run right after the
     # timed ones; "profiled": the timed steps themselves run the host loop
     # with an event pair around every kernel.
@@ -350,9 +350,9 @@ def run_ours(args) -> None:
         prof = G.get_profile()
         if args.trace:
             np.save(args.trace, G.get_trace())
-        # one more step with every exploit a single CUDA-graph launch and only
-        # the device-side trace on: how long the wave launches run, and the
-        # time between one launch's end and the next one's start
+        # one more step with every exploit a single launch and only the
+        # device-side trace on: how long its iterations run, and the time
+        # between one iteration's end and the next one's start
         G.set_profiling(2)
         graph_trace_ms, _, _ = timed_steps(1)
         gprof = G.get_profile()
@@ -460,7 +460,7 @@ def run_ours(args) -> None:
                                       2: "lane groups, FP32 screening", 1: "staged bulk copies",
                                       3: "lane groups, exact FP64"}[args.tile],
                    "improve_lanes_per_vertex": args.group or (4 if args.tile == 0 else 8),
-                   "timing": ("each exploit one CUDA-graph launch; per-kernel split and roofline "
+                   "timing": ("each exploit one launch; per-kernel split and roofline "
                               f"from {args.profile_steps} profiled step(s) (host loop, CUDA events "
                               f"around every kernel, {round(prof_ms / max(1, len(prof_times)), 3)} "
                               "ms per step) run right after the timed steps")
@@ -486,10 +486,9 @@ def run_ours(args) -> None:
             "step_ms": round(graph_trace_ms[0], 3), "wave_launches": gprof["wave_spans"],
             "wave_span_ms": round(gprof["wave_span_ns"] / 1e6, 3),
             "gaps": gprof["wave_gaps"], "gap_ms": round(gprof["wave_gap_ns"] / 1e6, 3),
-            "note": "one step of captured loops: wave launches from CTA 0's start to the end of "
-                    "their iteration, and the time from one launch's end to the next one's start "
-                    "within an exploit (the dense-sweep kernel between them and the launch "
-                    "latency), on the global timer"},
+            "note": "one step, every exploit one launch: iterations from CTA 0's start to their "
+                    "end, and the time from one iteration's end to the next one's start within "
+                    "an exploit, on the global timer"},
         "e2e": {"value": round(e2e_relax / e2e_s, 1) if e2e_steps else None, "unit": UNIT,
                 "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h),
                 "prefetch": not args.no_prefetch},
@@ -627,7 +626,7 @@ def openmp_baseline(rm, serial: dict, goal=None, h=None) -> dict:
 
 def run_batch(args) -> None:
     """Batched form: every member roadmap inserted and exploited to a fixpoint
-    in one CUDA-graph launch (options picked by the batch autotuner), next to
+    in one launch (options picked by the batch autotuner), next to
     the same members exploited one after another as separate graphs."""
     import torch
 

@@ -28,7 +28,7 @@
  *     it returns (its comment gives how long they must stay).
  *   - All device work is ordered on the stream given at create time
  *     (NULL = legacy default stream).  Calls that return results to the
- *     host (exploit, get_*) synchronise that stream before returning.
+ *     host (exploit, get_*) return when that stream's work has been done.
  *   - Errors are returned as pirrt_status; no exception crosses the ABI.
  *     Device kernels report errors through a status word, never by trapping.
  *     pirrt_graph_last_error() gives a human-readable detail string.
@@ -163,8 +163,8 @@ typedef struct pirrt_graph pirrt_graph;   /* opaque, library-owned */
  * row that outgrows it moves to the end of the pool, so an insertion copies
  * only the rows that moved; a second pool of the same size is allocated the
  * first time the pool is used up and every row is repacked -- plus 16 B of
- * row extent and about 130 B per vertex of
- * policy and work arrays.  *out is set to NULL on failure. */
+ * row extent and about 270 B per vertex of policy and work arrays (96 B of them
+ * the step lists and link records of the one-launch Replan loop).  *out is set to NULL on failure. */
 pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out);
 
 /* Free every allocation of the handle (NULL is ignored). */
@@ -419,7 +419,7 @@ pirrt_status pirrt_selftest_wait(int32_t which, int64_t limit, void *stream);
  * own root.  Policy iteration on the union is policy iteration on every
  * member at once (no edge joins two members), so every member reaches
  * exactly the policy of its own Replan, bit for bit; the whole batch runs in
- * one CUDA-graph launch per exploit.  Inserts are staged per member and
+ * one launch per exploit.  Inserts are staged per member and
  * merged into the device CSR in one pass at the next exploit (Sec. IV-A:
  * one CSR rebuild per Replan).
  * ------------------------------------------------------------------------ */

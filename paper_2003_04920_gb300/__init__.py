@@ -335,7 +335,7 @@ class Graph:
 
     def set_profiling(self, enable=True):
         """True: event timing (host loop); False: off; 2: the device-side wave
-        trace alone, every exploit still one CUDA-graph launch."""
+        trace alone, every exploit still one launch."""
         mode = 2 if enable == 2 else (1 if enable else 0)
         self._check("pirrt_graph_set_profiling",
                     self._lib.pirrt_graph_set_profiling(self._h, mode))
@@ -475,7 +475,7 @@ def exploit_opts(eps: float = 0.0, max_iters: int = 0, group: int = 0, tile: int
 class Batch:
     """Many independent planning graphs exploited together (wraps a
     ``pirrt_batch*``): the disjoint union of the members in one device graph,
-    one CUDA-graph launch per exploit."""
+    one launch per exploit."""
 
     def __init__(self, max_vertices, max_edges, roots=None, cost_dtype=np.float32,
                  device: int = 0, stream=None):

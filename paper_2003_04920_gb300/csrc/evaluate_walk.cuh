@@ -40,6 +40,7 @@ constexpr int kWalkSlots = 4;   // vertices a thread follows at once
 // any 32-bit vertex count, so vertices open after them lie below a cycle.
 constexpr int kWalkRounds = 16;
 constexpr int kWalkBarStride = 16;    // 64-bit words between barrier words
+constexpr size_t kWalkBarBytes = sizeof(unsigned long long) * kWalkBarStride * (kWalkRounds + 1);
 constexpr int kWalkMaxBlocks = 512;   // barrier words count to 1,023
 constexpr unsigned long long kWalkSpinLimit = 1ull << 22;
 
@@ -49,14 +50,18 @@ struct __align__(16) WalkRec {
     int32_t pad;
 };
 
+struct WalkBar {
+    unsigned long long *word;  // kWalkRounds + 1 barrier words, kWalkBarStride apart
+    unsigned long long call;   // number of this call: larger than any before it on these words
+};
+
 struct WalkArgs {
     const int32_t *parent;
     const double *cost;
     double *g;
     WalkRec *rec[2];
-    unsigned long long *bar;  // kWalkRounds + 1 barrier words, kWalkBarStride apart
+    WalkBar bar;
     unsigned *status;         // [0] outcome, [1] raised by a barrier that timed out
-    unsigned long long call;  // number of this call: larger than any before it on this device
     int64_t n;
     int32_t root;
 };
@@ -66,12 +71,12 @@ struct WalkArgs {
 // call's number above the counts (10 bits each, grids of at most kWalkMaxBlocks), so
 // it needs no clearing between calls: the first arrival of a call replaces
 // whatever an older one left.  Bounded: false after kWalkSpinLimit polls.
-__device__ __forceinline__ bool walk_sync(const WalkArgs &a, int k, bool open, bool bad,
+__device__ __forceinline__ bool walk_sync(const WalkBar &a, int k, bool open, bool bad,
                                           unsigned &n_open, unsigned &n_bad) {
     __shared__ unsigned s_open, s_bad, s_ok;
     const int o = __syncthreads_or(open), b = __syncthreads_or(bad);
     if (threadIdx.x == 0) {
-        unsigned long long *word = a.bar + kWalkBarStride * k;
+        unsigned long long *word = a.word + kWalkBarStride * k;
         const unsigned long long base = a.call << 30;
         atomicMax(word, base);
         const unsigned long long add = 1ull | (o ? 1ull << 10 : 0ull) | (b ? 1ull << 20 : 0ull);
@@ -83,7 +88,6 @@ __device__ __forceinline__ bool walk_sync(const WalkArgs &a, int k, bool open, b
             if (((unsigned)v & 1023u) == gridDim.x && (v >> 30) == a.call) break;
             if (++spins > kWalkSpinLimit) {
                 s_ok = 0u;
-                *reinterpret_cast<volatile unsigned *>(a.status + 1) = kStatusTimeout;
                 break;
             }
             __nanosleep(20);
@@ -97,40 +101,22 @@ __device__ __forceinline__ bool walk_sync(const WalkArgs &a, int k, bool open, b
     return s_ok != 0u;
 }
 
-static __global__ void __launch_bounds__(kWalkThreads, 1)
-walk_policy_kernel(const __grid_constant__ WalkArgs a) {
+// The rounds of a walk over the records rec[0] (and rec[1] for the vertices
+// finished at the start), written before the barrier in front.  done(v, g) takes
+// each vertex's g; a thread gets the vertices of a grid-stride loop.  False when a
+// barrier timed out; n_open > 0 afterwards: vertices below a cycle.
+template <typename Done>
+__device__ __forceinline__ bool walk_rounds(WalkRec *const (&rec)[2], int64_t n, const WalkBar &bar,
+                                            unsigned &n_open, const Done &done_with) {
     constexpr int K = kWalkSlots;
     const int64_t stride = (int64_t)gridDim.x * kWalkThreads;
     const int64_t t0 = (int64_t)blockIdx.x * kWalkThreads + threadIdx.x;
-    unsigned n_open = 0, n_bad = 0;
-
-    // Initial values, and the check of the policy before anything follows it:
-    // every parent is -1 or an id in [0, n), every used cost finite and >= 0.
-    bool bad = false;
-    for (int64_t v = t0; v < a.n; v += stride) {
-        const int32_t pv = a.parent[v];
-        const double c = a.cost[v];
-        const bool top = v == a.root || pv == -1;
-        WalkRec o;
-        o.pad = 0;
-        o.acc = v == a.root ? 0.0 : top ? CUDART_INF : c;
-        o.anc = top ? -2 : pv;
-        a.g[v] = v == a.root ? 0.0 : CUDART_INF;
-        a.rec[0][v] = o;
-        if (top) a.rec[1][v] = o;
-        else if (pv < 0 || (int64_t)pv >= a.n || !(c >= 0.0 && c <= DBL_MAX)) bad = true;
-    }
-    if (!walk_sync(a, 0, false, bad, n_open, n_bad)) return;
-    if (n_bad != 0u) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) a.status[0] = kStatusBadInput;
-        return;
-    }
-
+    unsigned none = 0;
     for (int r = 1;; ++r) {
-        const WalkRec *rd = a.rec[(r - 1) & 1];
-        WalkRec *wr = a.rec[r & 1];
+        const WalkRec *rd = rec[(r - 1) & 1];
+        WalkRec *wr = rec[r & 1];
         bool open = false;
-        for (int64_t base = t0; base < a.n; base += K * stride) {
+        for (int64_t base = t0; base < n; base += K * stride) {
             double s[K], low[K], end[K];
             int32_t x[K];
             unsigned work = 0, done = 0;
@@ -139,7 +125,7 @@ walk_policy_kernel(const __grid_constant__ WalkArgs a) {
                 const int64_t v = base + k * stride;
                 x[k] = -2;
                 s[k] = low[k] = end[k] = 0.0;
-                if (v < a.n) {
+                if (v < n) {
                     const int4 q = __ldcg(reinterpret_cast<const int4 *>(rd + v));
                     x[k] = q.z;
                     s[k] = __hiloint2double(q.y, q.x);
@@ -183,7 +169,7 @@ walk_policy_kernel(const __grid_constant__ WalkArgs a) {
                 if ((done >> k) & 1u) {
                     o.acc = s[k] + end[k];
                     o.anc = -1;
-                    a.g[v] = o.acc;
+                    done_with(v, o.acc);
                 } else if ((mine >> k) & 1u) {
                     open = true;
                 } else if (x[k] == -1) {
@@ -194,10 +180,43 @@ walk_policy_kernel(const __grid_constant__ WalkArgs a) {
                 wr[v] = o;
             }
         }
-        if (!walk_sync(a, r, open, false, n_open, n_bad)) return;
-        if (n_open == 0u || r == kWalkRounds) break;
+        if (!walk_sync(bar, r, open, false, n_open, none)) return false;
+        if (n_open == 0u || r == kWalkRounds) return true;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.status[0] = n_open ? kStatusBadTree : 0u;
+}
+
+static __global__ void __launch_bounds__(kWalkThreads, 1)
+walk_policy_kernel(const __grid_constant__ WalkArgs a) {
+    const int64_t stride = (int64_t)gridDim.x * kWalkThreads;
+    const int64_t t0 = (int64_t)blockIdx.x * kWalkThreads + threadIdx.x;
+    unsigned n_open = 0, n_bad = 0;
+
+    // Initial values, and the check of the policy before anything follows it:
+    // every parent is -1 or an id in [0, n), every used cost finite and >= 0.
+    bool bad = false;
+    for (int64_t v = t0; v < a.n; v += stride) {
+        const int32_t pv = a.parent[v];
+        const double c = a.cost[v];
+        const bool top = v == a.root || pv == -1;
+        WalkRec o;
+        o.pad = 0;
+        o.acc = v == a.root ? 0.0 : top ? CUDART_INF : c;
+        o.anc = top ? -2 : pv;
+        a.g[v] = v == a.root ? 0.0 : CUDART_INF;
+        a.rec[0][v] = o;
+        if (top) a.rec[1][v] = o;
+        else if (pv < 0 || (int64_t)pv >= a.n || !(c >= 0.0 && c <= DBL_MAX)) bad = true;
+    }
+    bool ok = walk_sync(a.bar, 0, false, bad, n_open, n_bad);
+    if (ok && n_bad != 0u) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.status[0] = kStatusBadInput;
+        return;
+    }
+
+    ok = ok && walk_rounds(a.rec, a.n, a.bar, n_open, [&](int64_t v, double g) { a.g[v] = g; });
+    if (threadIdx.x != 0) return;
+    if (!ok) *reinterpret_cast<volatile unsigned *>(a.status + 1) = kStatusTimeout;
+    else if (blockIdx.x == 0) a.status[0] = n_open ? kStatusBadTree : 0u;
 }
 
 }  // namespace pirrt

@@ -1274,50 +1274,6 @@ static __global__ void set_roots_kernel(int64_t k, const int32_t *__restrict__ r
     }
 }
 
-// ---------------------------------------------------------------------------
-// Policy replacement (set_policy): look up each parent edge's cost.
-// ---------------------------------------------------------------------------
-
-template <typename CT>
-__global__ void __launch_bounds__(kThreads)
-policy_lookup_kernel(int64_t n, int32_t root, const int32_t *__restrict__ parent,
-                     const RowExt *__restrict__ rows, const Entry<CT> *__restrict__ adj,
-                     int32_t *__restrict__ p_out, CT *__restrict__ pc_out, DevCounters *c) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t q = parent[v];
-        if (v == root) {
-            if (q != -1) atomicOr(&c->status, kStatusBadInput);
-            p_out[v] = kRootMark;
-            pc_out[v] = CT(0);
-            continue;
-        }
-        if (q == -1) {
-            p_out[v] = -1;
-            pc_out[v] = CT(0);
-            continue;
-        }
-        if (q < 0 || q >= n) {
-            atomicOr(&c->status, kStatusBadInput);
-            continue;
-        }
-        bool found = false;
-        CT best = CT(0);
-        int64_t rb, re;
-        row_range(rows, v, rb, re);
-        for (int64_t i = rb; i < re; ++i) {
-            const Entry<CT> en = adj[i];
-            if (en.col == q && (!found || en.w < best)) {
-                best = en.w;
-                found = true;
-            }
-        }
-        if (!found) atomicOr(&c->status, kStatusBadInput);
-        p_out[v] = q;
-        pc_out[v] = best;
-    }
-}
-
 // Restore (checkpoint load): packed rows from their offsets, no room to grow
 // yet; the FP32 shadow from g; no pending offers.
 static __global__ void __launch_bounds__(kThreads)
@@ -1333,21 +1289,6 @@ restore_rows(int64_t n, const int64_t *__restrict__ off, RowExt *__restrict__ ro
         rows[v] = r;
         g32[v] = g32_of(g[v]);
         cand[v] = kCandNone;
-    }
-}
-
-// Commit a looked-up policy and clear g (Evaluate refills it).
-template <typename CT>
-__global__ void __launch_bounds__(kThreads)
-policy_commit_kernel(int64_t n, int32_t root, const int32_t *__restrict__ p_in,
-                     const CT *__restrict__ pc_in, int32_t *__restrict__ p, CT *__restrict__ pc,
-                     double *__restrict__ g, float *__restrict__ g32) {
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x) {
-        p[v] = p_in[v];
-        pc[v] = pc_in[v];
-        g[v] = (v == root) ? 0.0 : CUDART_INF;
-        g32[v] = (v == root) ? 0.0f : __int_as_float(0x7f800000);
     }
 }
 

@@ -29,6 +29,7 @@
 #include "replan_iteration.cuh"
 #include "insert.cuh"
 #include "replan_loop.cuh"
+#include "set_policy.cuh"
 #include "pirrt.h"
 
 using namespace pirrt;
@@ -67,6 +68,8 @@ struct pirrt_graph {
     int64_t *hx = nullptr;         // pinned host scalars read back by insertion
     InsertReport *insert_rep = nullptr;  // pinned: what an insertion's kernel tells the host
     unsigned insert_seq = 0;
+    unsigned long long *walk_words = nullptr;  // set_policy: barrier words, numbered calls
+    unsigned long long walk_calls = 0;
     HostSignal *sig = nullptr;           // pinned: the end of a read-back, or of a batch insert
     unsigned sig_seq = 0;
     int insert_blocks = 0;               // co-resident grid of the insertion kernel
@@ -124,7 +127,8 @@ struct pirrt_graph {
     size_t stage_bytes = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     WaveItem *items[2] = {nullptr, nullptr};  // persistent loop: grid-step lists
-    JumpRec *rec[2] = {nullptr, nullptr};     // ... pointer-jumping records
+    JumpRec *rec[2] = {nullptr, nullptr};     // ... pointer-jumping records (also set_policy's)
+    static_assert(sizeof(JumpRec) == sizeof(WalkRec), "one array serves both");
     LoopResult *loop_res = nullptr;           // ... what an exploit reports (pinned)
     int loop_occ = 0;                         // ... CTAs per SM (<= 2)
     int eval_blocks = 0;
@@ -1153,31 +1157,39 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
 
 template <typename CT>
 pirrt_status set_policy_impl(pirrt_graph *G, const int32_t *parent) {
-    // look up into scratch (anc[0] for ids, acc[1] reinterpreted for costs)
-    int32_t *tp = G->anc[0];
-    CT *tc = reinterpret_cast<CT *>(G->acc[1]);
-    const int blocks = grid_for(G->n, kThreads, G->num_sms * 32);
-    CK(cudaMemsetAsync(&G->ctr->status, 0, sizeof(unsigned), G->stream));
-    policy_lookup_kernel<CT><<<blocks, kThreads, 0, G->stream>>>(
-        G->n, G->cfg.root, parent, G->rows, static_cast<const Entry<CT> *>(G->adj[G->cur]),
-        tp, tc, G->ctr);
-    CKL();
-    CK(cudaMemcpyAsync(&G->ctr_host->status, &G->ctr->status, sizeof(unsigned),
-                       cudaMemcpyDeviceToHost, G->stream));
-    CK(cudaStreamSynchronize(G->stream));
-    if (G->ctr_host->status) {
-        CK(cudaMemsetAsync(&G->ctr->status, 0, sizeof(unsigned), G->stream));
+    PolicyArgs<CT> a{};
+    a.n = G->n;
+    a.root = G->cfg.root;
+    a.parent = parent;
+    a.rows = G->rows;
+    a.adj = static_cast<const Entry<CT> *>(G->adj[G->cur]);
+    a.p = G->p;
+    a.pc = static_cast<CT *>(G->pc);
+    a.g = G->g;
+    a.g32 = G->g32;
+    for (int k = 0; k < 2; ++k) a.rec[k] = reinterpret_cast<WalkRec *>(G->rec[k]);
+    a.bar.word = G->walk_words;
+    a.bar.call = ++G->walk_calls;
+    a.ctr = G->ctr;
+    a.host = G->sig;
+    a.seq = ++G->sig_seq;
+    const int blocks = grid_for(8 * G->n, kWalkThreads, std::min(G->num_sms, kWalkMaxBlocks));
+    void *args[] = {&a};
+    CK(cudaLaunchCooperativeKernel((const void *)set_policy_kernel<CT>, dim3(blocks),
+                                   dim3(kWalkThreads), args, 0, G->stream));
+    if (const pirrt_status rc = wait_host(G, &G->sig->seq, a.seq)) return rc;
+    if (G->sig->status & kStatusBadInput)
         return fail(G, PIRRT_ERR_BAD_INPUT,
                     "set_policy: parent out of range, root with a parent, or a parent edge not in G");
-    }
-    policy_commit_kernel<CT><<<blocks, kThreads, 0, G->stream>>>(
-        G->n, G->cfg.root, tp, tc, G->p, static_cast<CT *>(G->pc), G->g, G->g32);
+    if (const pirrt_status rc = status_from_bits(G, G->sig->status)) return rc;
+    begin_exploit_kernel<<<1, 1, 0, G->stream>>>(G->ctr, 1u, 0ull);
     CKL();
-    return reevaluate_impl<CT>(G);
+    G->stale = 0;
+    return PIRRT_OK;
 }
 
 // Evaluate the whole policy tree (pointer jumping, no pruning) and make the
-// next Improve sweep every vertex: after set_policy, and in the goal-directed
+// next Improve sweep every vertex: after a device timeout, and in the goal-directed
 // form after the goal or h changed, since subtrees pruned for the old goal
 // may hold values that are not up to date.
 template <typename CT>
@@ -1231,7 +1243,7 @@ void free_all(pirrt_graph *G) {
                     G->deg, G->tile_sums, G->stamp, G->list[0], G->list[1], G->switched,
                     G->dg, G->anc[0], G->anc[1], G->acc[0], G->acc[1], G->wx[0], G->wx[1], G->done, G->wl[0],
                     G->wl[1], G->wstamp, G->swstamp, G->cand, G->aq, G->aring, G->ctr, G->stage, G->h,
-                    G->items[0], G->items[1], G->rec[0], G->rec[1]};
+                    G->items[0], G->items[1], G->rec[0], G->rec[1], G->walk_words};
     for (void *q : bufs)
         if (q) cudaFree(q);
     if (G->ctr_host) cudaFreeHost(G->ctr_host);
@@ -1436,6 +1448,8 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     ALLOC(G->ctr, sizeof(DevCounters));
     ALLOC(G->dargs, kArgBytes);
     ALLOC(G->pexport, sizeof(int32_t) * nv);
+    ALLOC(G->walk_words, kWalkBarBytes);
+    if (cudaMemset(G->walk_words, 0, kWalkBarBytes) != cudaSuccess) return bail(PIRRT_ERR_CUDA);
     for (int k = 0; k < 2; ++k) {
         ALLOC(G->items[k], sizeof(WaveItem) * nv);
         ALLOC(G->rec[k], sizeof(JumpRec) * nv);

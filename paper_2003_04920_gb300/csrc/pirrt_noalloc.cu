@@ -31,8 +31,7 @@ constexpr int64_t kMaxNoAllocVertices = 1 << 18;  // 262,144
 
 // Two records per vertex, a line per barrier and one for the outcome: 8.4 MB.
 constexpr size_t kRecBytes = sizeof(WalkRec) * (size_t)kMaxNoAllocVertices;
-constexpr size_t kBarBytes = sizeof(unsigned long long) * kWalkBarStride * (kWalkRounds + 1);
-constexpr size_t kScratchBytes = 2 * kRecBytes + kBarBytes + 256;
+constexpr size_t kScratchBytes = 2 * kRecBytes + kWalkBarBytes + 256;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -99,14 +98,14 @@ extern "C" pirrt_status pirrt_evaluate_noalloc(int64_t n, int32_t root, const in
     a.g = g_out;
     a.rec[0] = reinterpret_cast<WalkRec *>(s.scratch);
     a.rec[1] = reinterpret_cast<WalkRec *>(s.scratch + kRecBytes);
-    a.bar = reinterpret_cast<unsigned long long *>(s.scratch + 2 * kRecBytes);
-    a.call = s.calls.fetch_add(1) + 1;
+    a.bar.word = reinterpret_cast<unsigned long long *>(s.scratch + 2 * kRecBytes);
+    a.bar.call = s.calls.fetch_add(1) + 1;
     a.n = n;
     a.root = root;
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned *const dev_outcome =
-        reinterpret_cast<unsigned *>(s.scratch + 2 * kRecBytes + kBarBytes);
+        reinterpret_cast<unsigned *>(s.scratch + 2 * kRecBytes + kWalkBarBytes);
     volatile unsigned *outcome = g_outcome[dev];
     unsigned copied[2];
     outcome[0] = kNoOutcome;
