@@ -34,19 +34,21 @@
 // warps and a CTA barrier between the phases the tensor core waited for each
 // of them: 10^6 rows over 32 scenes took 418 us, now 163.
 //
-// What bounds it is the data path of shared memory and L1, which MMA operands
-// and the epilogues share (100 % busy, the tensor core 33 %, FP32 units 23 %), so
-// the layouts below are chosen to move fewer bytes over it.  Both accumulators are
-// read as 16 lanes x 32 columns, which gives a thread several columns of four
-// rows instead of many columns of one: a row's scene terms then arrive as whole
-// 128-byte lines (a thread per row: one 16-byte piece of 32 different lines a
-// load, 250 us a call against 225), and b2 and W3 are read once for four rows.
-// The accumulators' columns are permuted (column_unit: in the weights' rows, at
-// no cost) so that a thread's eight are consecutive.  N = 256 instructions read H
-// once instead of twice (225 -> 209 us a call together with two-wide FP32
-// arithmetic).  Tried and slower: a second register set for the next block's
-// sums (233 - 267 us, spills), a loading warp (227), layer 2 in two column
-// halves with early release of the accumulator (212 - 223).
+// What bounds it is the path that MMA operands, gathers and epilogues share into
+// shared memory and L1, and the chain between the roles: the MMAs alone take 1.44 us
+// a tile, with either epilogue beside them 2.4, with both 2.9.  The layouts below are
+// chosen to move fewer bytes (that path was 100 % busy before the last of these
+// steps, 62 % after).  Both accumulators are read as 16 lanes x 32 columns, which
+// gives a thread several columns of four rows instead of many columns of one: a
+// row's scene terms then arrive as whole 128-byte lines (a thread per row: one
+// 16-byte piece of 32 different lines a load, 250 us a call against 225), and b2
+// and W3 are read once for four rows.  The accumulators' columns are permuted
+// (column_unit: in the weights' rows, at no cost) so that a thread's eight are
+// consecutive.  N = 256 instructions read H once instead of twice (225 -> 209 us a
+// call together with two-wide FP32 arithmetic).  Tried and slower: a second
+// register set for the next block's sums (233 - 267 us, spills), a loading warp
+// (213 - 227), layer 2 in two column halves with early release of the accumulator
+// (212 - 223).
 //
 // Every wait is bounded.  A wait that expires ends every other wait of its CTA at
 // once, so the roles run to the end without waiting for one another and issue no
