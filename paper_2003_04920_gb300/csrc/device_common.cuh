@@ -146,6 +146,8 @@ struct DevCounters {
     alignas(128) unsigned wl_count[kMaxJumpRounds + 2];  // pointer-jumping work-list sizes per round
     alignas(128) unsigned n_touched;   // insertion: old rows gaining entries (list length)
     unsigned insert_status;            // ... kStatus* bits
+    unsigned insert_late;              // ... a barrier timed out: rows may name entries never
+                                       // written, so nothing follows the CSR until a reset
     alignas(128) unsigned sig_ticket;  // signal_host: CTAs done
     unsigned sig_status;               // ... kStatus* bits to tell the host
     alignas(128) unsigned long long pool_cursor;  // insertion: pool room taken by the block

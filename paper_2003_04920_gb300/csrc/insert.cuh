@@ -40,7 +40,6 @@ struct InsertReport {
     unsigned long long need;  // pool room the block takes
     unsigned status;          // kStatus* bits
     unsigned seq;             // number of the insertion
-    unsigned late;            // a barrier timed out after the report (stays set)
 };
 
 template <typename CT>
@@ -346,24 +345,32 @@ __device__ __forceinline__ void insert_report(const InsertArgs<CT> &a, unsigned 
     r->seq = a.seq;
 }
 
+// A barrier timed out here: later launches see it whatever this one reports.
+__device__ __forceinline__ unsigned insert_gave_up(DevCounters *c) {
+    if (threadIdx.x == 0) atomicExch(&c->insert_late, 1u);
+    return kStatusTimeout;
+}
+
 template <typename CT>
 __global__ void __launch_bounds__(kInsertThreads, 3)
 insert_kernel(const __grid_constant__ InsertArgs<CT> a) {
     __shared__ unsigned long long s_scan[kInsertThreads / 32 + 2];
     DevCounters *c = a.ctr;
+    // (set by an earlier launch, or past this one's first barrier)
+    if (__ldcg(&c->insert_late) != 0u) return insert_report<CT>(a, kStatusTimeout);
     insert_count<CT>(a, s_scan);
-    if (!grid_barrier(c, gridDim.x)) return insert_report<CT>(a, kStatusTimeout);
+    if (!grid_barrier(c, gridDim.x)) return insert_report<CT>(a, insert_gave_up(c));
     const unsigned status = __ldcg(&c->insert_status);
     if (status != 0u) return insert_report<CT>(a, status);
     const int64_t nt = (int64_t)__ldcg(&c->n_touched);
     insert_room<CT>(a, nt, s_scan);
-    if (!grid_barrier(c, gridDim.x)) return insert_report<CT>(a, kStatusTimeout);
+    if (!grid_barrier(c, gridDim.x)) return insert_report<CT>(a, insert_gave_up(c));
     insert_report<CT>(a, 0u);
     if (a.pool_used + (long long)__ldcg(&c->pool_cursor) > a.pool_cap) return;
     insert_move<CT>(a, nt);
     insert_init<CT>(a);
     if (!grid_barrier(c, gridDim.x)) {
-        if (threadIdx.x == 0) *const_cast<volatile unsigned *>(&a.report->late) = 1u;
+        insert_gave_up(c);
         return;
     }
     insert_entries<CT>(a, s_scan);

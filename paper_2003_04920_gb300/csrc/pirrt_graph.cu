@@ -68,6 +68,8 @@ struct pirrt_graph {
     int64_t *hx = nullptr;         // pinned host scalars read back by insertion
     InsertReport *insert_rep = nullptr;  // pinned: what an insertion's kernel tells the host
     unsigned insert_seq = 0;
+    int insert_open = 0;                 // its end has not been waited for (insertion_ended)
+    int bar_dirty = 0;                   // a barrier timed out: its word may be part-way
     unsigned long long *walk_words = nullptr;  // set_policy: barrier words, numbered calls
     unsigned long long walk_calls = 0;
     HostSignal *sig = nullptr;           // pinned: the end of a read-back, or of a batch insert
@@ -175,7 +177,10 @@ int grid_for(int64_t work, int threads, int max_blocks) {
 }
 
 pirrt_status status_from_bits(pirrt_graph *G, unsigned bits) {
-    if (bits & kStatusTimeout) return fail(G, PIRRT_ERR_DEVICE_TIMEOUT, "grid barrier timed out");
+    if (bits & kStatusTimeout) {
+        G->bar_dirty = 1;
+        return fail(G, PIRRT_ERR_DEVICE_TIMEOUT, "grid barrier timed out");
+    }
     if (bits & kStatusBadTree) return fail(G, PIRRT_ERR_BAD_TREE, "parent pointers contain a cycle");
     if (bits & kStatusBadInput) return fail(G, PIRRT_ERR_BAD_INPUT, "invalid input rejected on device");
     return PIRRT_OK;
@@ -680,6 +685,19 @@ pirrt_status insert_plan_scan(pirrt_graph *G, int64_t n_old, int64_t n_after, in
     return PIRRT_OK;
 }
 
+// The kernels outside the one-launch loop do not look at insert_late: the host does,
+// once after insertions.
+pirrt_status insertion_ended(pirrt_graph *G) {
+    if (!G->insert_open) return PIRRT_OK;
+    CK(cudaMemcpyAsync(&G->ctr_host->insert_late, &G->ctr->insert_late, sizeof(unsigned),
+                       cudaMemcpyDeviceToHost, G->stream));
+    CK(cudaStreamSynchronize(G->stream));
+    if (G->ctr_host->insert_late)
+        return fail(G, PIRRT_ERR_DEVICE_TIMEOUT, "insert_batch: a grid barrier timed out");
+    G->insert_open = 0;
+    return PIRRT_OK;
+}
+
 template <typename CT>
 pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const int32_t *src,
                          const int32_t *dst, const CT *cost) {
@@ -717,6 +735,11 @@ pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const i
         a.ctr = G->ctr;
         a.report = rep;
         // no more CTAs than the block keeps busy: a barrier costs its arrivals
+        if (G->bar_dirty) {
+            insert_clear_kernel<<<1, 1, 0, G->stream>>>(G->ctr);
+            CKL();
+            G->bar_dirty = 0;
+        }
         const int64_t items = std::max<int64_t>((n_edges + kInsertUnroll - 1) / kInsertUnroll, n_new);
         const int blocks = grid_for(items, kInsertThreads, G->insert_blocks);
         void *args[] = {&a};
@@ -725,7 +748,8 @@ pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const i
         // the report comes before the entries are written
         if (const pirrt_status rc = wait_host(G, &rep->seq, a.seq)) return rc;
         G->prof.launches += 1;
-        if (rep->status || rep->late) {
+        G->insert_open = 1;
+        if (rep->status) {
             insert_clear_kernel<<<1, 1, 0, G->stream>>>(G->ctr);
             CKL();
             CK(cudaMemsetAsync(G->deg, 0, sizeof(int32_t) * (size_t)(n_after + 1), G->stream));
@@ -992,9 +1016,11 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
         (sizeof(CT) == 8 || gs == 0 || gs == 4))
         return exploit_loop<CT>(G, o, jump, mode == PIRRT_EVAL_AUTO && !small,
                                 small ? kTopRounds : 0, max_iters, dense_limit, max_levels, st);
-    pirrt_status rc = write_args<CT>(G, dense_limit, max_levels, tile == 0 ? 1 : 0, tail_max,
-                                     local_levels, local_max, local_step);
+    pirrt_status rc = insertion_ended(G);
     if (rc) return rc;
+    if ((rc = write_args<CT>(G, dense_limit, max_levels, tile == 0 ? 1 : 0, tail_max, local_levels,
+                             local_max, local_step)))
+        return rc;
     const int wave_ctas = o.wave_ctas > 0 ? std::min(o.wave_ctas, G->wave_occ) : G->wave_occ;
     G->wave_blocks = G->num_sms * wave_ctas;
     const bool prof = G->profiling != 0;
@@ -1743,8 +1769,6 @@ pirrt_status pirrt_graph_exploit(pirrt_graph *G, const pirrt_exploit_opts *opts,
     const pirrt_status rc = G->cfg.cost_dtype == PIRRT_COST_F32 ? exploit_impl<float>(G, opts, stats)
                                                                 : exploit_impl<double>(G, opts, stats);
     if (rc != PIRRT_OK) G->async_dirty = 1;
-    if (rc == PIRRT_OK && *const_cast<volatile unsigned *>(&G->insert_rep->late))
-        return fail(G, PIRRT_ERR_DEVICE_TIMEOUT, "insert_batch: a grid barrier timed out");
     return rc;
 }
 

@@ -1288,7 +1288,11 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
     bool walk = a.walk != 0;  // ... until a policy is too deep for it
     LoopCounters *ic = &c->loop[par];
     __syncthreads();
-    if (sizeof(CT) == 4 && dense && stale) {
+    if (vld(&c->insert_late) != 0u) {  // an insertion did not end: its rows are not followed
+        ok = false;
+        if (tid == 0) atomicOr(&c->status, kStatusTimeout);
+    }
+    if (sizeof(CT) == 4 && ok && dense && stale) {
         for (int64_t v = (int64_t)blockIdx.x * kLoopThreads + tid; v < a.n;
              v += (int64_t)gridDim.x * kLoopThreads)
             a.g32[v] = g32_of(__ldcg(&a.g[v]));
