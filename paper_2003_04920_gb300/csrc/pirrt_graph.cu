@@ -998,7 +998,11 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
     // jumping; probe with a wave again every eighth exploit
     bool jump = mode == PIRRT_EVAL_JUMP ||
                 (mode == PIRRT_EVAL_AUTO && G->deep_hint && (G->exploits % 8) != 0);
-    const bool small = mode == PIRRT_EVAL_AUTO && G->goal < 0 &&
+    const bool one_launch = G->profiling != 1 && o.host_loop == 0 && tile == 0 && !async &&
+                            (sizeof(CT) == 8 || gs == 0 || gs == 4);
+    // (its pointer jumping only: the other forms' costs more than their wave up to
+    // twice, 17.0 against 9.9 ms on 150,000 vertices in 2-D with tile 2)
+    const bool small = one_launch && mode == PIRRT_EVAL_AUTO && G->goal < 0 &&
                        G->n <= (sizeof(CT) == 8 ? kJumpVerticesF64 : kJumpVertices);
     if (small) jump = true;
     G->exploits += 1;
@@ -1012,8 +1016,7 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
         o.wave_local < 0 ? 0u : (o.wave_local > 0 ? (unsigned)o.wave_local : 32u);
     const unsigned local_max = o.wave_local_max > 0 ? (unsigned)o.wave_local_max : 128u;
     const unsigned local_step = o.wave_local_step > 0 ? (unsigned)o.wave_local_step : 4096u;
-    if (G->profiling != 1 && o.host_loop == 0 && tile == 0 && !async &&
-        (sizeof(CT) == 8 || gs == 0 || gs == 4))
+    if (one_launch)
         return exploit_loop<CT>(G, o, jump, mode == PIRRT_EVAL_AUTO && !small,
                                 small ? kTopRounds : 0, max_iters, dense_limit, max_levels, st);
     pirrt_status rc = insertion_ended(G);
