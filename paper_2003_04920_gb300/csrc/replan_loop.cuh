@@ -1020,8 +1020,11 @@ __device__ __forceinline__ bool loop_jump(const LoopArgs<CT> &a, LoopCounters *i
 // sum runs from itself upwards, as in loop_jump; with FP64 costs, whose sums
 // round, the links are kept on a stack and added from the root down, as Alg. 2
 // adds them, up to the depth that top_round covers.  A vertex deeper than that, or
-// below a cycle, sends the whole Evaluate to loop_jump, which finds the others
-// as it would leave them (and the rest of the exploit goes there at once).
+// below a cycle, sends the whole Evaluate to loop_jump (and the rest of the exploit
+// goes there at once): every CTA first puts back what it wrote and the list of
+// changed vertices starts empty, because pointer jumping may round the same sums
+// differently, and a vertex listed by both would not fit the list, which has room
+// for each vertex once.
 // At most 128 vertices a CTA (64 with stacks): with one warp per scheduler the
 // slow FP64 additions hide behind the loads.
 //
@@ -1137,6 +1140,13 @@ __device__ __forceinline__ bool loop_walk(const LoopArgs<CT> &a, LoopCounters *i
     if (!loop_sync<CT>(a.ctr, sh, left)) return false;
     if (sh.total != 0u) {
         walk = false;
+        if (changed) {
+            a.g[v] = old;
+            a.g32[v] = g32_of(old);
+        }
+        // (every append came before the barrier above, loop_jump's come after the next)
+        if (blockIdx.x == 0 && threadIdx.x == 0) ic->n_jump = 0u;
+        if (!loop_sync<CT>(a.ctr, sh, 0u)) return false;
         return loop_jump<CT>(a, ic, stale);
     }
     if (threadIdx.x == 0) {
