@@ -358,6 +358,8 @@ insert_kernel(const __grid_constant__ InsertArgs<CT> a) {
     DevCounters *c = a.ctr;
     // (set by an earlier launch, or past this one's first barrier)
     if (__ldcg(&c->insert_late) != 0u) return insert_report<CT>(a, kStatusTimeout);
+    // what an earlier exploit reported does not stop the next one
+    if (blockIdx.x == 0 && threadIdx.x == 0) c->status = 0u;
     insert_count<CT>(a, s_scan);
     if (!grid_barrier(c, gridDim.x)) return insert_report<CT>(a, insert_gave_up(c));
     const unsigned status = __ldcg(&c->insert_status);

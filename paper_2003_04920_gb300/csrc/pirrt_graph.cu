@@ -811,6 +811,8 @@ pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const i
             }
             G->prof.launches += 6 + (n_new > 0) + (n_edges > 0);
         }
+    } else {
+        CK(cudaMemsetAsync(&G->ctr->status, 0, sizeof(unsigned), G->stream));
     }
     G->prof.insert_calls += 1;
     G->prof.insert_new_entries += 2 * n_edges;

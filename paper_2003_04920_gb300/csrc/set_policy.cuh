@@ -98,6 +98,7 @@ set_policy_kernel(const __grid_constant__ PolicyArgs<CT> a) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned status = !ok ? kStatusTimeout : n_bad ? kStatusBadInput
                                 : n_open ? kStatusBadTree : 0u;
+        a.ctr->status = 0u;  // what an earlier exploit found wrong is replaced
         if (status == 0u) {
             a.ctr->dense = 1u;  // the next Improve sweeps every vertex; the seeded list is moot
             a.ctr->g32_stale = 0u;
