@@ -4,7 +4,9 @@
 // Looking up was one thread per vertex going through its row alone, and the steps
 // took seven launches and three waits of the host.  Here eight lanes share a row,
 // the costs found are the evaluation's first records, nothing is written to the
-// graph before every vertex has passed the check, and the host polls one word.
+// graph before every vertex's parent edge has passed the check (a cycle shows in the
+// evaluation only: it is reported, and again by an exploit), and the host polls one
+// word.
 // What bounds it is the row reads for large graphs, the barriers and the host's
 // part of the call for small ones.  2,000 vertices with FP64 costs: a call 102 us
 // before, 31 now.
@@ -98,7 +100,9 @@ set_policy_kernel(const __grid_constant__ PolicyArgs<CT> a) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned status = !ok ? kStatusTimeout : n_bad ? kStatusBadInput
                                 : n_open ? kStatusBadTree : 0u;
-        a.ctr->status = 0u;  // what an earlier exploit found wrong is replaced
+        // what an earlier exploit found wrong is replaced; a policy that was committed
+        // and could not be evaluated stops the next one
+        a.ctr->status = status & (kStatusBadTree | kStatusTimeout);
         if (status == 0u) {
             a.ctr->dense = 1u;  // the next Improve sweeps every vertex; the seeded list is moot
             a.ctr->g32_stale = 0u;

@@ -1,5 +1,5 @@
-"""After an exploit that met a cycle in the parents: a valid policy or an insertion
-takes the error away, as a reset does."""
+"""A cycle in the parents: set_policy reports it, and so does every exploit until a
+valid policy or an insertion takes the error away, as a reset does."""
 import numpy as np
 import pytest
 
@@ -57,3 +57,21 @@ def test_a_valid_policy_or_an_insertion_recovers(n, dtype):
     d, _ = O.dijkstra(n, np.r_[u, 0].astype(np.int32), np.r_[v, n - 1].astype(np.int32),
                       np.r_[c.astype(np.float64), 0.25])
     np.testing.assert_allclose(got, d, rtol=n * 2.0 ** -52, atol=0)
+
+
+@pytest.mark.parametrize("kw", [{}, dict(evaluate="wave"), dict(evaluate="jump"),
+                                dict(host_loop=True)])
+def test_an_exploit_over_a_rejected_policy_reports_it(kw):
+    n = 60
+    u, v, c, par, loop = _path(n, np.float32)
+    with P.Graph(n - 1, n, 0, np.float32) as G:
+        G.insert_batch(n - 1, u, v, c)
+        G.set_policy(par)
+        G.exploit()
+        want = G.get_costs()
+        assert _status(G.set_policy, loop) == P.PIRRT_ERR_BAD_TREE
+        for _ in range(2):
+            assert _status(G.exploit, **kw) == P.PIRRT_ERR_BAD_TREE
+        G.set_policy(par)
+        assert G.exploit(**kw)["converged"] == 1
+        np.testing.assert_array_equal(G.get_costs(), want)
