@@ -411,6 +411,13 @@ pirrt_status pirrt_evaluate_noalloc(int64_t n, int32_t root, const int32_t *pare
 enum { PIRRT_SELFTEST_GRID_BARRIER = 0, PIRRT_SELFTEST_MBARRIER = 1 };
 pirrt_status pirrt_selftest_wait(int32_t which, int64_t limit, void *stream);
 
+/* The same for what follows such a wait: leaves the graph as an insertion does
+ * whose last barrier timed out, after which rows may name entries that were never
+ * written.  From then on every call that follows rows (insert_batch, set_policy,
+ * exploit, save, get_adjacency) returns PIRRT_ERR_DEVICE_TIMEOUT, until
+ * pirrt_graph_reset or pirrt_graph_load.  Synchronises the graph's stream. */
+pirrt_status pirrt_selftest_insert_timeout(pirrt_graph *g);
+
 /* ------------------------------------------------------------------------
  * Batched form: many independent planning graphs exploited together.
  *

@@ -149,6 +149,7 @@ def load_library(path: str = LIB_PATH):
         "pirrt_status_string": (ctypes.c_char_p, [st]),
         "pirrt_evaluate_noalloc": (st, [i64, ctypes.c_int32, vp, vp, vp, vp]),
         "pirrt_selftest_wait": (st, [ctypes.c_int32, i64, vp]),
+        "pirrt_selftest_insert_timeout": (st, [vp]),
         "pirrt_batch_create": (st, [ctypes.c_int32, vp, vp, vp, ctypes.c_int32, ctypes.c_int32, vp,
                                     ctypes.POINTER(vp)]),
         "pirrt_batch_destroy": (None, [vp]),
@@ -390,6 +391,12 @@ class Graph:
     def load(self, path: str):
         """Replace this graph's contents with a checkpoint."""
         self._check("pirrt_graph_load", self._lib.pirrt_graph_load(self._h, os.fsencode(path)))
+
+    def selftest_insert_timeout(self):
+        """Leave the graph as an insertion does whose barrier timed out (failure
+        detection self-test): calls that follow rows fail until a reset."""
+        self._check("pirrt_selftest_insert_timeout",
+                    self._lib.pirrt_selftest_insert_timeout(self._h))
 
 
 def pirrt_status_string(status: int) -> str:

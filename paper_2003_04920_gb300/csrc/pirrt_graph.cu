@@ -685,8 +685,9 @@ pirrt_status insert_plan_scan(pirrt_graph *G, int64_t n_old, int64_t n_after, in
     return PIRRT_OK;
 }
 
-// The kernels outside the one-launch loop do not look at insert_late: the host does,
-// once after insertions.
+// Insertion, set_policy and the one-launch loop look at insert_late themselves.  For
+// every other launch that follows rows (the other loop forms, get_adjacency, save)
+// the host does, once after insertions.
 pirrt_status insertion_ended(pirrt_graph *G) {
     if (!G->insert_open) return PIRRT_OK;
     CK(cudaMemcpyAsync(&G->ctr_host->insert_late, &G->ctr->insert_late, sizeof(unsigned),
@@ -2042,6 +2043,7 @@ pirrt_status pirrt_graph_save(const pirrt_graph *Gc, const char *path) {
     pirrt_graph *G = const_cast<pirrt_graph *>(Gc);
     if (!G || !path) return PIRRT_ERR_INVALID_ARG;
     CK(cudaSetDevice(G->cfg.device));
+    if (const pirrt_status rc = insertion_ended(G)) return rc;  // before a file is overwritten
     FILE *f = std::fopen(path, "wb");
     if (!f) return fail(G, PIRRT_ERR_INVALID_ARG, "save: cannot open %s", path);
     const pirrt_status rc = G->cfg.cost_dtype == PIRRT_COST_F32 ? save_impl<float>(G, f)
@@ -2078,10 +2080,21 @@ pirrt_status pirrt_graph_get_adjacency(const pirrt_graph *Gc, int64_t *row_off, 
     pirrt_graph *G = const_cast<pirrt_graph *>(Gc);
     if (!G) return PIRRT_ERR_INVALID_ARG;
     CK(cudaSetDevice(G->cfg.device));
+    if (const pirrt_status rc = insertion_ended(G)) return rc;
     if (G->cfg.cost_dtype == PIRRT_COST_F32) return export_impl<float>(G, row_off, col, cost, on_device);
     return export_impl<double>(G, row_off, col, cost, on_device);
 }
 
+pirrt_status pirrt_selftest_insert_timeout(pirrt_graph *G) {
+    if (!G) return PIRRT_ERR_INVALID_ARG;
+    CK(cudaSetDevice(G->cfg.device));
+    const unsigned one = 1u;
+    CK(cudaMemcpyAsync(&G->ctr->insert_late, &one, sizeof(unsigned), cudaMemcpyHostToDevice,
+                       G->stream));
+    CK(cudaStreamSynchronize(G->stream));
+    G->insert_open = 1;
+    return PIRRT_OK;
+}
 
 pirrt_status pirrt_batch_create(int32_t n_graphs, const int64_t *max_vertices,
                                 const int64_t *max_edges, const int32_t *roots,

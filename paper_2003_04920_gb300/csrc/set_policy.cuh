@@ -42,6 +42,15 @@ set_policy_kernel(const __grid_constant__ PolicyArgs<CT> a) {
     const int lane = threadIdx.x & 31, gl = lane & (L - 1);
     unsigned n_open = 0, n_bad = 0;
     bool bad = false;
+    if (__ldcg(&a.ctr->insert_late) != 0u) {  // an insertion did not end: its rows are not followed
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            volatile HostSignal *h = a.host;
+            h->status = kStatusTimeout;
+            __threadfence_system();
+            h->seq = a.seq;
+        }
+        return;
+    }
 
     // the cheapest edge to the parent, for parallel edges
     const int64_t warps = (int64_t)gridDim.x * (kWalkThreads / 32);
