@@ -220,9 +220,11 @@ bool own_memory(const pirrt_graph *G, const void *p) {
     return at.type == cudaMemoryTypeDevice && at.device == G->cfg.device;
 }
 
-// n costs from `from` into the caller's buffer, complete on return.
+// n costs from `from` into the caller's buffer, complete on return.  A copy takes any
+// address; the kernel's stores need their 8 bytes aligned.
 pirrt_status costs_out(pirrt_graph *G, const double *from, double *out, int64_t n, int on_device) {
-    if (n > 0 && on_device && own_memory(G, out)) {
+    const bool aligned = reinterpret_cast<uintptr_t>(out) % sizeof(double) == 0;
+    if (n > 0 && on_device && aligned && own_memory(G, out)) {
         export_costs_kernel<<<grid_for(n, kThreads, G->num_sms * 8), kThreads, 0, G->stream>>>(
             n, from, out, G->ctr, G->sig, ++G->sig_seq);
         CKL();
