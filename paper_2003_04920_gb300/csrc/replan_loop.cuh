@@ -1357,7 +1357,12 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
             if (!jump) {
                 // ---- Evaluate, top-down in grid steps
                 int64_t count = (int64_t)n_sw;
+                bool lost = false;
                 for (unsigned t = 0;; ++t) {
+                    // a vertex lowered several times in a step (parallel edges)
+                    // takes as many entries: those past the end of the list are
+                    // lost, and with them the offers of their vertices.  Pointer
+                    // jumping finishes every value; the next sweep is dense.
                     const bool stop = count > a.list_cap;
                     if (stop) count = a.list_cap;
                     if (tid == 0) {
@@ -1384,6 +1389,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
                                              !walk ? 0u : tail ? 0xffffffffu : a.local_levels,
                                              tail ? kStage : a.local_max);
                     ok = loop_sync<CT>(c, sh, made);
+                    lost = stop;
                     if (!ok || stop) break;
                     count = (int64_t)sh.total;
                     if (count == 0) break;
@@ -1391,7 +1397,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
                 if (!ok) break;
                 loop_fetch<CT>(c, ic, sh);
                 if (tid == 0) trace_step(c, sh.tr, 0, 0);
-                next_dense = sh.v_ndg > a.dense_limit;
+                next_dense = lost || sh.v_ndg > a.dense_limit;
                 next_count = sh.v_next;
                 jump = (sh.v_flags & kLoopIncomplete) != 0u;
                 stale = true;
