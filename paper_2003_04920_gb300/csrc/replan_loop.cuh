@@ -1297,6 +1297,14 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
     bool converged = false, ok = true;
     bool walk = a.walk != 0;  // ... until a policy is too deep for it
     LoopCounters *ic = &c->loop[par];
+    if (blockIdx.x == 0 && tid == 0) {
+        // the other loop forms leave their totals behind (this one's are added
+        // after its barriers)
+        c->relax = 0ull;
+        c->improved = 0ull;
+        c->evaluated = 0ull;
+        c->offers = 0ull;
+    }
     __syncthreads();
     if (vld(&c->insert_late) != 0u) {  // an insertion did not end: its rows are not followed
         ok = false;
@@ -1500,10 +1508,6 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
             r.jump_rounds = __ldcg(&c->loop_state.jump_rounds);
             r.jump_evals = __ldcg(&c->loop_state.jump_evals);
             *a.res = r;
-            c->relax = 0ull;
-            c->improved = 0ull;
-            c->evaluated = 0ull;
-            c->offers = 0ull;
         }
     }
 }
