@@ -42,7 +42,6 @@ constexpr int kWalkRounds = 16;
 constexpr int kWalkBarStride = 16;    // 64-bit words between barrier words
 constexpr size_t kWalkBarBytes = sizeof(unsigned long long) * kWalkBarStride * (kWalkRounds + 1);
 constexpr int kWalkMaxBlocks = 512;   // barrier words count to 1,023
-constexpr unsigned long long kWalkSpinLimit = 1ull << 22;
 
 struct __align__(16) WalkRec {
     double acc;   // cost up to anc; g once anc < 0
@@ -70,7 +69,7 @@ struct WalkArgs {
 // sees the last arrival holds how many CTAs raised each.  The word carries the
 // call's number above the counts (10 bits each, grids of at most kWalkMaxBlocks), so
 // it needs no clearing between calls: the first arrival of a call replaces
-// whatever an older one left.  Bounded: false after kWalkSpinLimit polls.
+// whatever an older one left.  Bounded: false after kBarrierSpinLimit polls.
 __device__ __forceinline__ bool walk_sync(const WalkBar &a, int k, bool open, bool bad,
                                           unsigned &n_open, unsigned &n_bad) {
     __shared__ unsigned s_open, s_bad, s_ok;
@@ -86,7 +85,7 @@ __device__ __forceinline__ bool walk_sync(const WalkBar &a, int k, bool open, bo
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
             if (((unsigned)v & 1023u) == gridDim.x && (v >> 30) == a.call) break;
-            if (++spins > kWalkSpinLimit) {
+            if (++spins > kBarrierSpinLimit) {
                 s_ok = 0u;
                 break;
             }

@@ -37,7 +37,6 @@ constexpr int kLoopWarps = kLoopThreads / 32;
 constexpr unsigned kChunk = kLoopThreads;  // vertices a CTA takes from a list at a time
 constexpr unsigned kStage = 768;     // lowered children staged per CTA
 constexpr unsigned kMarkCap = 2048;  // Improve-list appends staged per CTA
-constexpr unsigned long long kLoopSpinLimit = 1ull << 22;  // barrier polls: seconds
 
 // A vertex to expand: its row [beg, beg + len), the lowered g it carries and its
 // depth below the switched vertex it came from.
@@ -170,7 +169,7 @@ __device__ __forceinline__ bool loop_sync(DevCounters *c, LoopShared<CT> &sh, un
             v = ld_acquire(word);
             // arrivals, modulo 2^24
             if ((((unsigned)(v >> 40) - target) & 0x800000u) == 0u) break;
-            if (++spins > kLoopSpinLimit) {
+            if (++spins > kBarrierSpinLimit) {
                 atomicOr(&c->status, kStatusTimeout);
                 ok = 0u;
                 break;
