@@ -1004,7 +1004,7 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
     bool jump = mode == PIRRT_EVAL_JUMP ||
                 (mode == PIRRT_EVAL_AUTO && G->deep_hint && (G->exploits % 8) != 0);
     const bool one_launch = G->profiling != 1 && o.host_loop == 0 && tile == 0 && !async &&
-                            (sizeof(CT) == 8 || gs == 0 || gs == 4);
+                            (gs == 0 || gs == (sizeof(CT) == 8 ? 8 : 4));
     // (its pointer jumping only: the other forms' costs more than their wave up to
     // twice, 17.0 against 9.9 ms on 150,000 vertices in 2-D with tile 2)
     const bool small = one_launch && mode == PIRRT_EVAL_AUTO && G->goal < 0 &&
