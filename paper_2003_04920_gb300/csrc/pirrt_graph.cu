@@ -2349,7 +2349,7 @@ std::vector<TuneDim> tune_dims(int32_t cost_dtype) {
                  [](pirrt_exploit_opts &o, double v) { o.wave_local = (int32_t)v; }});
     d.push_back({"wave_local_max", {32, 128, 512},
                  [](pirrt_exploit_opts &o, double v) { o.wave_local_max = (int32_t)v; }});
-    d.push_back({"wave_local_step", {1024, 4096, 16384},
+    d.push_back({"wave_local_step", {512, 1024, 4096, 16384},
                  [](pirrt_exploit_opts &o, double v) { o.wave_local_step = (int32_t)v; }});
     d.push_back({"wave_tail", {-1, 64, 256},
                  [](pirrt_exploit_opts &o, double v) { o.wave_tail = (int32_t)v; }});
@@ -2370,14 +2370,17 @@ pirrt_status pirrt_batch_autotune_search(pirrt_batch *B, const pirrt_exploit_opt
     pirrt_exploit_opts cur{};
     if (start) cur = *start;
     // the defaults, written out, so that each coordinate starts from a value
-    // of its list
-    if (cur.group == 0) cur.group = 4;
+    // of its list (the one-launch loop's walk differs from the other forms')
+    const int lanes = G->cfg.cost_dtype == PIRRT_COST_F32 ? 4 : 8;
+    const bool loop = cur.tile == 0 && (cur.group == 0 || cur.group == lanes) &&
+                      cur.evaluate != PIRRT_EVAL_ASYNC && cur.host_loop == 0;
+    if (cur.group == 0) cur.group = lanes;
     if (cur.dense_fraction == 0.0) cur.dense_fraction = 0.35;
     if (cur.wave_ctas == 0) cur.wave_ctas = 2;
     if (cur.wave_local == 0) cur.wave_local = 32;
-    if (cur.wave_local_max == 0) cur.wave_local_max = 128;
-    if (cur.wave_local_step == 0) cur.wave_local_step = 4096;
-    if (cur.wave_tail == 0) cur.wave_tail = 64;
+    if (cur.wave_local_max == 0) cur.wave_local_max = loop ? 32 : 128;
+    if (cur.wave_local_step == 0) cur.wave_local_step = loop ? 512 : 4096;
+    if (cur.wave_tail == 0) cur.wave_tail = loop ? -1 : 64;
     const std::vector<TuneDim> dims = tune_dims(G->cfg.cost_dtype);
     TrialRunner tr(B);
     pirrt_status rc = tr.begin();
