@@ -92,16 +92,18 @@ struct LoopArgs {
 };
 
 // What a grid step's warps share.
+constexpr unsigned kStepOffersOnly = 1u;  // the list overflowed: no children
+constexpr unsigned kStepTraced = 2u;      // this CTA's tiles are traced
 struct StepView {
     int32_t *next;
     WaveItem *out;
     unsigned *out_cnt;
     unsigned tag, epoch;
-    bool nochild;  // the list overflowed: offers only
+    unsigned flags;
 };
 
 struct LoopTrace {
-    long long t;
+    long long t, tile;
     unsigned long long ns0;
     int state;  // -1 off, -2 between steps, b >= 0 the running step's bucket
 };
@@ -527,7 +529,8 @@ __device__ __forceinline__ void expand(const LoopArgs<CT> &a, LoopShared<CT> &sh
                                        bool offering, unsigned &recomputed, unsigned &first) {
     const unsigned lane = threadIdx.x & 31u;
     const int gl = (int)(lane & (unsigned)(L - 1));
-    const bool nochild = s.nochild || (unsigned)it.depth >= a.max_levels;
+    const bool nochild =
+        (s.flags & kStepOffersOnly) != 0u || (unsigned)it.depth >= a.max_levels;
     const int32_t u = nochild ? INT_MIN : it.u;  // no parent: every neighbour is offered to
     const int depth = it.depth + 1, len = it.len;
     const Entry<CT> *row = a.adj + it.beg;
@@ -699,6 +702,72 @@ __device__ __forceinline__ void step_flush(const LoopArgs<CT> &a, LoopShared<CT>
     __syncthreads();
 }
 
+// Level trace of CTA 0's thread 0 while tracing (profile fields level_*,
+// share_*, local_*, wave_*): a grid step's cycles run from its start to the next
+// one's, a tile's from its start to the barrier that ends it.
+__device__ __forceinline__ unsigned long long loop_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+__device__ __forceinline__ void trace_iteration(DevCounters *c, LoopTrace &tr, unsigned iter) {
+    if (tr.state == -1) return;
+    tr.state = -2;
+    tr.t = clock64();
+    const unsigned long long now = loop_ns();
+    if (iter > 0u) {
+        c->gap_ns += now - tr.ns0;  // tr.ns0: end of the iteration before
+        c->gaps += 1ull;
+    }
+    tr.ns0 = now;
+}
+
+__device__ __forceinline__ void trace_step(DevCounters *c, LoopTrace &tr, long long count) {
+    if (tr.state == -1) return;
+    const long long now = clock64();
+    const unsigned long long d = (unsigned long long)(now - tr.t);
+    if (tr.state == -2) c->ph_pre_cyc += d;
+    else {
+        c->lvl_cyc[tr.state] += d;
+    }
+    tr.t = now;
+    tr.state = -2;
+    if (count > 0) {
+        int b = 64 - __clzll((unsigned long long)count);
+        if (b >= kLevelBuckets) b = kLevelBuckets - 1;
+        c->lvl_n[b] += 1ull;
+        c->lvl_items[b] += (unsigned long long)count;
+        tr.state = b;
+    }
+}
+
+// A tile of nv vertices (its start in shared memory: a register held across the
+// expansion spills).
+__device__ __forceinline__ void trace_tile_start(LoopTrace &tr) {
+    if (threadIdx.x == 0) tr.tile = clock64();
+}
+__device__ __forceinline__ void trace_tile(LoopTrace &tr, unsigned long long *n,
+                                           unsigned long long *items, unsigned long long *cyc,
+                                           unsigned nv) {
+    if (threadIdx.x != 0) return;
+    int b = 32 - __clz(nv);
+    if (b >= kLevelBuckets) b = kLevelBuckets - 1;
+    n[b] += 1ull;
+    items[b] += (unsigned long long)nv;
+    cyc[b] += (unsigned long long)(clock64() - tr.tile);
+}
+
+__device__ __forceinline__ void trace_end(DevCounters *c, LoopTrace &tr) {
+    if (tr.state == -1) return;
+    c->ph_post_cyc += (unsigned long long)(clock64() - tr.t);
+    const unsigned long long now = loop_ns();
+    c->span_ns += now - tr.ns0;
+    c->spans += 1ull;
+    c->ph_calls += 1ull;
+    tr.ns0 = now;
+}
+
 // One CTA's part of a grid step: its share [lo, hi) of the step's list, a chunk
 // at a time, then, where `levels` allows, the lowered children on its own, tree
 // level by tree level, while there are at most `limit` of them.  What is left
@@ -711,6 +780,7 @@ __device__ __forceinline__ unsigned loop_step(const LoopArgs<CT> &a, LoopCounter
     const StepView s = sh.step;
     unsigned cur = 0;
     for (int64_t c0 = lo; c0 < hi; c0 += kChunk) {
+        if (s.flags & kStepTraced) trace_tile_start(sh.tr);
         const unsigned n = hi - c0 < (int64_t)kChunk ? (unsigned)(hi - c0) : kChunk;
         unsigned gone = 0;
         if (threadIdx.x < n) {
@@ -737,11 +807,13 @@ __device__ __forceinline__ unsigned loop_step(const LoopArgs<CT> &a, LoopCounter
             }
             sh.item[cur][threadIdx.x] = it;
         }
-        if (s.nochild && threadIdx.x == 0) sh.incomplete = 1u;
+        if ((s.flags & kStepOffersOnly) && threadIdx.x == 0) sh.incomplete = 1u;
         if (switched && threadIdx.x == 0) sh.tot[2] += n;
         __syncthreads();
         expand_stage<CT>(a, sh, ic, s, cur, n);
         __syncthreads();
+        if (s.flags & kStepTraced)
+            trace_tile(sh.tr, a.ctr->shr_n, a.ctr->shr_items, a.ctr->shr_cyc, n);
         if (c0 + kChunk < hi && (sh.nitem[cur ^ 1u] > kStage / 2 || sh.nmark > kMarkCap / 2))
             step_flush<CT>(a, sh, ic, s, cur ^ 1u,
                            sh.nitem[cur ^ 1u] < kStage ? sh.nitem[cur ^ 1u] : kStage);
@@ -749,10 +821,13 @@ __device__ __forceinline__ unsigned loop_step(const LoopArgs<CT> &a, LoopCounter
     for (unsigned l = 0;; ++l) {
         const unsigned m = sh.nitem[cur ^ 1u], n = m < kStage ? m : kStage;
         if (n == 0u || l >= levels || m > limit) break;
+        if (s.flags & kStepTraced) trace_tile_start(sh.tr);
         cur ^= 1u;
         __syncthreads();  // every thread has read the count
         expand_stage<CT>(a, sh, ic, s, cur, n);
         __syncthreads();
+        if (s.flags & kStepTraced)
+            trace_tile(sh.tr, a.ctr->loc_n, a.ctr->loc_items, a.ctr->loc_cyc, n);
         if (threadIdx.x == 0) sh.nitem[cur] = 0u;
     }
     const unsigned k = cur ^ 1u, m = sh.nitem[k];
@@ -1211,62 +1286,6 @@ __device__ __forceinline__ void loop_mark(const LoopArgs<CT> &a, LoopCounters *i
     flush_marks<CT>(sh, next, &ic->n_next);
 }
 
-// Level trace of CTA 0's thread 0 while tracing (profile fields level_*,
-// share_*, wave_*): a grid step's cycles run from its start to the next one's.
-__device__ __forceinline__ unsigned long long loop_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void trace_iteration(DevCounters *c, LoopTrace &tr, unsigned iter) {
-    if (tr.state == -1) return;
-    tr.state = -2;
-    tr.t = clock64();
-    const unsigned long long now = loop_ns();
-    if (iter > 0u) {
-        c->gap_ns += now - tr.ns0;  // tr.ns0: end of the iteration before
-        c->gaps += 1ull;
-    }
-    tr.ns0 = now;
-}
-
-__device__ __forceinline__ void trace_step(DevCounters *c, LoopTrace &tr, long long count,
-                                           long long share) {
-    if (tr.state == -1) return;
-    const long long now = clock64();
-    const unsigned long long d = (unsigned long long)(now - tr.t);
-    if (tr.state == -2) c->ph_pre_cyc += d;
-    else {
-        c->lvl_cyc[tr.state] += d;
-    }
-    tr.t = now;
-    tr.state = -2;
-    if (count > 0) {
-        int b = 64 - __clzll((unsigned long long)count);
-        if (b >= kLevelBuckets) b = kLevelBuckets - 1;
-        c->lvl_n[b] += 1ull;
-        c->lvl_items[b] += (unsigned long long)count;
-        if (share > 0) {
-            int sb = 64 - __clzll((unsigned long long)share);
-            if (sb >= kLevelBuckets) sb = kLevelBuckets - 1;
-            c->shr_n[sb] += 1ull;
-            c->shr_items[sb] += (unsigned long long)share;
-        }
-        tr.state = b;
-    }
-}
-
-__device__ __forceinline__ void trace_end(DevCounters *c, LoopTrace &tr) {
-    if (tr.state == -1) return;
-    c->ph_post_cyc += (unsigned long long)(clock64() - tr.t);
-    const unsigned long long now = loop_ns();
-    c->span_ns += now - tr.ns0;
-    c->spans += 1ull;
-    c->ph_calls += 1ull;
-    tr.ns0 = now;
-}
-
 template <typename CT>
 __global__ void __launch_bounds__(kLoopThreads, 1)
 replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
@@ -1284,7 +1303,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
     }
     if (tid == 0) {
         sh.tr.state = (blockIdx.x == 0 && c->lvl_trace != 0u) ? -2 : -1;
-        sh.tr.t = 0;
+        sh.tr.t = sh.tr.tile = 0;
         sh.tr.ns0 = 0ull;
     }
     // loop state, the same in every CTA; CTA 0 writes it back at the end
@@ -1358,7 +1377,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
         bool next_dense = false;
         unsigned levels = 0;
         int32_t *next = la ? a.list[0] : a.list[1];
-        if (tid == 0 && (n_sw == 0u || a.jump != 0)) trace_step(c, sh.tr, 0, 0);
+        if (tid == 0 && (n_sw == 0u || a.jump != 0)) trace_step(c, sh.tr, 0);
         if (n_sw != 0u) {
             bool jump = a.jump != 0;
             if (!jump) {
@@ -1378,7 +1397,8 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
                         sh.step.out_cnt = &ic->wave_cnt[(t + 1u) % 3u];
                         sh.step.tag = tag;
                         sh.step.epoch = epoch + 1u;
-                        sh.step.nochild = stop;
+                        sh.step.flags = (stop ? kStepOffersOnly : 0u) |
+                                        (sh.tr.state != -1 ? kStepTraced : 0u);
                     }
                     __syncthreads();
                     const bool tail = count <= (int64_t)a.tail_max;
@@ -1388,7 +1408,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
                                            ? (int64_t)blockIdx.x * per : count;
                     const int64_t hi = lo + per < count ? lo + per : count;
                     if (blockIdx.x == 0 && tid == 0) ic->wave_cnt[(t + 2u) % 3u] = 0u;
-                    if (tid == 0) trace_step(c, sh.tr, count, hi - lo);
+                    if (tid == 0) trace_step(c, sh.tr, count);
                     ++levels;
                     unsigned made = 0;
                     if (lo < hi)
@@ -1403,7 +1423,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
                 }
                 if (!ok) break;
                 loop_fetch<CT>(c, ic, sh);
-                if (tid == 0) trace_step(c, sh.tr, 0, 0);
+                if (tid == 0) trace_step(c, sh.tr, 0);
                 next_dense = lost || sh.v_ndg > a.dense_limit;
                 next_count = sh.v_next;
                 jump = (sh.v_flags & kLoopIncomplete) != 0u;
