@@ -72,6 +72,13 @@ def load():
     lib.rgg_edges.restype = ctypes.c_int
     lib.rgg_edges.argtypes = [i32, i64, vp, i32, vp, i32, vp, vp, i32, i32, i32, vp, vp, vp, vp,
                               i64, vp, vp]
+    lib.rgg_links_mark.restype = ctypes.c_int
+    lib.rgg_links_mark.argtypes = [i32, i64, vp, i32, vp, i32, vp, vp, i32, i32, vp, vp, vp,
+                                   ctypes.POINTER(vp)]
+    lib.rgg_links_fill.restype = ctypes.c_int
+    lib.rgg_links_fill.argtypes = [vp, i32, vp, vp, vp, vp]
+    lib.rgg_links_destroy.restype = None
+    lib.rgg_links_destroy.argtypes = [vp]
     _lib = lib
     return lib
 
@@ -132,19 +139,22 @@ def edges(points, nbr, scene: Scene, exact_segment: bool, n_check: int = 16,
     tdt = torch.float64 if f64 else torch.float32
     start = torch.empty(n + 1, dtype=torch.int64, device="cuda")
     m = ctypes.c_int64(0)
-    # room for every link (a second pass over the links to count them first would
-    # cost as much as the first); the result is a view of its used part
-    cap = n * k
-    u = torch.empty(cap, dtype=torch.int32, device="cuda")
-    v = torch.empty(cap, dtype=torch.int32, device="cuda")
-    cost = torch.empty(cap, dtype=tdt, device="cuda")
-    _check("rgg_edges", lib.rgg_edges(dim, n, points.data_ptr(), k, nbr.data_ptr(),
-                                      len(scene.radii), c.data_ptr(), r.data_ptr(),
-                                      0 if exact_segment else 1, int(n_check), 1 if f64 else 0,
-                                      u.data_ptr(), v.data_ptr(), cost.data_ptr(),
-                                      start.data_ptr(), cap, ctypes.byref(m), _stream()))
-    mm = int(m.value)
-    return u[:mm], v[:mm], cost[:mm], start.cpu().numpy()
+    h, stream = ctypes.c_void_p(), _stream()
+    _check("rgg_links_mark", lib.rgg_links_mark(dim, n, points.data_ptr(), k, nbr.data_ptr(),
+                                                len(scene.radii), c.data_ptr(), r.data_ptr(),
+                                                0 if exact_segment else 1, int(n_check),
+                                                start.data_ptr(), ctypes.byref(m), stream,
+                                                ctypes.byref(h)))
+    try:
+        mm = int(m.value)
+        u = torch.empty(mm, dtype=torch.int32, device="cuda")
+        v = torch.empty(mm, dtype=torch.int32, device="cuda")
+        cost = torch.empty(mm, dtype=tdt, device="cuda")
+        _check("rgg_links_fill", lib.rgg_links_fill(h, 1 if f64 else 0, u.data_ptr(),
+                                                    v.data_ptr(), cost.data_ptr(), stream))
+    finally:
+        lib.rgg_links_destroy(h)
+    return u, v, cost, start.cpu().numpy()
 
 
 @dataclass

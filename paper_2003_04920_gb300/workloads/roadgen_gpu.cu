@@ -6,6 +6,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <memory>
+#include <new>
 #include <type_traits>
 #include <vector>
 
@@ -877,57 +879,89 @@ extern "C" int rgg_knn(int32_t dim, double lo, double hi, int64_t n, const doubl
     return 0;
 }
 
-extern "C" int rgg_edges(int32_t dim, int64_t n, const double *points, int32_t k,
-                         const int32_t *knn, int32_t n_obs, const double *centers,
-                         const double *radii, int32_t mode, int32_t n_check, int32_t cost_f64,
-                         int32_t *u, int32_t *v, void *cost, int64_t *edge_start, int64_t cap,
-                         int64_t *m, void *stream) {
+// What marking the links leaves for writing them.
+struct rgg_links {
+    int dim = 0, k = 0;
+    long long n = 0, total = 0;
+    const double *points = nullptr;
+    const int *knn = nullptr;
+    const long long *vstart = nullptr;
+    Arena w;
+    unsigned *keep = nullptr;
+    int *vcnt = nullptr;
+    bool filled = false;  // the cursors have moved
+};
+
+extern "C" void rgg_links_destroy(rgg_links *x) { delete x; }
+
+extern "C" int rgg_links_mark(int32_t dim, int64_t n, const double *points, int32_t k,
+                              const int32_t *knn, int32_t n_obs, const double *centers,
+                              const double *radii, int32_t mode, int32_t n_check,
+                              int64_t *edge_start, int64_t *m, void *stream, rgg_links **out) {
+    if (!out) return 1;
+    *out = nullptr;
     if (dim < 1 || dim > kMaxDim || n < 1 || k < 1 || !points || !knn || !edge_start || !m ||
         (mode != 0 && mode != 1) || (mode == 1 && n_check < 1) || n_obs < 0 ||
         (n_obs > 0 && (!centers || !radii)))
         return 1;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    std::unique_ptr<rgg_links> x(new (std::nothrow) rgg_links);
+    if (!x) return 2;
     const size_t words = (size_t)(k + 31) / 32;
-    Arena w;
+    Arena &w = x->w;
     const size_t o_keep = w.add<unsigned>((size_t)n * words), o_vcnt = w.add<int>(n + 1),
                  o_tiles = w.add<long long>((n + 1) / kTile + 2),
                  o_obs = w.add<float>((size_t)n_obs * (dim + 2));
     if (!w.alloc()) return 2;
-    unsigned *keep = w.at<unsigned>(o_keep);
-    int *vcnt = w.at<int>(o_vcnt);
+    x->dim = dim;
+    x->k = k;
+    x->n = n;
+    x->points = points;
+    x->knn = knn;
+    x->keep = w.at<unsigned>(o_keep);
+    x->vcnt = w.at<int>(o_vcnt);
     long long *tiles = w.at<long long>(o_tiles), *vstart = reinterpret_cast<long long *>(edge_start);
+    x->vstart = vstart;
     float *obs = w.at<float>(o_obs);
     if (n_obs > 0) {
         obstacles_f32<<<(n_obs + kT - 1) / kT, kT, 0, st>>>(n_obs, dim, centers, radii, obs);
         RG_CKL();
     }
-    RG_CK(cudaMemsetAsync(vcnt, 0, sizeof(int) * (n + 1), st));
+    RG_CK(cudaMemsetAsync(x->vcnt, 0, sizeof(int) * (n + 1), st));
     with_dim(dim, [&](auto D) {
         edge_mark<decltype(D)::value><<<grid_of(n * 32), kT, 0, st>>>(
-            n, points, k, knn, n_obs, obs, centers, radii, mode, n_check, keep, vcnt);
+            n, points, k, knn, n_obs, obs, centers, radii, mode, n_check, x->keep, x->vcnt);
     });
     RG_CKL();
-    if (int rc = exclusive_scan(vcnt, n + 1, vstart, tiles, st)) return rc;
-    long long total = 0;
-    RG_CK(cudaMemcpyAsync(&total, vstart + n, sizeof(total), cudaMemcpyDeviceToHost, st));
-    RG_CK(cudaMemsetAsync(vcnt, 0, sizeof(int) * (n + 1), st));  // now the groups' cursors
+    if (int rc = exclusive_scan(x->vcnt, n + 1, vstart, tiles, st)) return rc;
+    RG_CK(cudaMemcpyAsync(&x->total, vstart + n, sizeof(x->total), cudaMemcpyDeviceToHost, st));
+    RG_CK(cudaMemsetAsync(x->vcnt, 0, sizeof(int) * (n + 1), st));  // now the groups' cursors
     RG_CK(cudaStreamSynchronize(st));
-    *m = total;
-    if (total > cap || (total > 0 && (!u || !v || !cost))) return total > cap ? 3 : 1;
+    *m = x->total;
+    *out = x.release();
+    return 0;
+}
+
+extern "C" int rgg_links_fill(rgg_links *x, int32_t cost_f64, int32_t *u, int32_t *v, void *cost,
+                              void *stream) {
+    if (!x || x->filled || (x->total > 0 && (!u || !v || !cost))) return 1;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const long long n = x->n;
     Arena t;
-    const size_t o_u = t.add<int>(total);
-    const size_t o_c = cost_f64 ? t.add<double>(total) : t.add<float>(total);
+    const size_t o_u = t.add<int>(x->total);
+    const size_t o_c = cost_f64 ? t.add<double>(x->total) : t.add<float>(x->total);
     if (!t.alloc()) return 2;
+    x->filled = true;
     int *tu = t.at<int>(o_u);
     const auto fill = [&](auto zero) {
         using CT = decltype(zero);
         CT *tc = t.at<CT>(o_c);
-        with_dim(dim, [&](auto D) {
+        with_dim(x->dim, [&](auto D) {
             edge_fill<decltype(D)::value, CT><<<grid_of(n * 32), kT, 0, st>>>(
-                n, points, k, knn, keep, vstart, vcnt, tu, tc);
+                n, x->points, x->k, x->knn, x->keep, x->vstart, x->vcnt, tu, tc);
         });
         RG_CKL();
-        group_sort<CT><<<grid_of(n * 32), kT, 0, st>>>(n, vstart, tu, tc, u, v,
+        group_sort<CT><<<grid_of(n * 32), kT, 0, st>>>(n, x->vstart, tu, tc, u, v,
                                                        static_cast<CT *>(cost));
         RG_CKL();
         return 0;
@@ -935,6 +969,20 @@ extern "C" int rgg_edges(int32_t dim, int64_t n, const double *points, int32_t k
     if (const int rc = cost_f64 ? fill(0.0) : fill(0.f)) return rc;
     RG_CK(cudaStreamSynchronize(st));
     return 0;
+}
+
+extern "C" int rgg_edges(int32_t dim, int64_t n, const double *points, int32_t k,
+                         const int32_t *knn, int32_t n_obs, const double *centers,
+                         const double *radii, int32_t mode, int32_t n_check, int32_t cost_f64,
+                         int32_t *u, int32_t *v, void *cost, int64_t *edge_start, int64_t cap,
+                         int64_t *m, void *stream) {
+    rgg_links *x = nullptr;
+    if (const int rc = rgg_links_mark(dim, n, points, k, knn, n_obs, centers, radii, mode, n_check,
+                                      edge_start, m, stream, &x))
+        return rc;
+    const std::unique_ptr<rgg_links> own(x);
+    if (x->total > cap) return 3;
+    return rgg_links_fill(x, cost_f64, u, v, cost, stream);
 }
 
 // ---- incremental exploration ------------------------------------------------

@@ -65,6 +65,19 @@ int rgg_edges(int32_t dim, int64_t n, const double *points, int32_t k, const int
               int32_t n_check, int32_t cost_f64, int32_t *u, int32_t *v, void *cost,
               int64_t *edge_start, int64_t cap, int64_t *m, void *stream);
 
+/* rgg_edges in two steps, for buffers of exactly the edge count: mark finds the
+ * edges, writes edge_start and *m and returns a handle; fill writes them (once) into
+ * u, v and cost of m entries each.  points, knn and edge_start stay as they are until
+ * then.  Destroy frees the handle's workspace (NULL is ignored). */
+typedef struct rgg_links rgg_links;
+int rgg_links_mark(int32_t dim, int64_t n, const double *points, int32_t k, const int32_t *knn,
+                   int32_t n_obs, const double *centers, const double *radii, int32_t mode,
+                   int32_t n_check, int64_t *edge_start, int64_t *m, void *stream,
+                   rgg_links **out);
+int rgg_links_fill(rgg_links *x, int32_t cost_f64, int32_t *u, int32_t *v, void *cost,
+                   void *stream);
+void rgg_links_destroy(rgg_links *x);
+
 /* Incremental exploration: the Extend step of RRT# one Batched-Extension
  * block at a time (Alg. 3), for running on its own stream while the previous
  * block is exploited (the asynchronous exploration the paper leaves to future
