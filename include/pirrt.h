@@ -163,8 +163,9 @@ typedef struct pirrt_graph pirrt_graph;   /* opaque, library-owned */
  * row that outgrows it moves to the end of the pool, so an insertion copies
  * only the rows that moved; a second pool of the same size is allocated the
  * first time the pool is used up and every row is repacked -- plus 16 B of
- * row extent and about 270 B per vertex of policy and work arrays (96 B of them
- * the step lists and link records of the one-launch Replan loop).  *out is set to NULL on failure. */
+ * row extent and about 180 B per vertex of policy and work arrays (96 B of them one
+ * block that insertions, exploits and read-backs use in turn).  *out is set to NULL
+ * on failure. */
 pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out);
 
 /* Free every allocation of the handle (NULL is ignored). */

@@ -19,6 +19,7 @@
 #include <map>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "evaluate_async.cuh"
@@ -61,6 +62,10 @@ struct pirrt_graph {
     void *adj[2] = {nullptr, nullptr};  // pools; the second is allocated on the first repack
     int64_t pool_cap = 0;          // entries per pool
     int64_t pool_used = 0;         // entries taken in the live pool (rows, slack, moved-out)
+    void *scratch = nullptr;       // holds nothing between calls: one block for the arrays of
+                                   // insertion and export (ralloc, touched, roff, pexport), of
+                                   // the one-launch loop and set_policy (items, rec), and of
+                                   // the other loop forms (switched .. wl)
     int32_t *ralloc = nullptr;     // insertion: pool space per row
     int32_t *touched = nullptr;    // insertion: old rows gaining entries
     int64_t *roff = nullptr;       // insertion / export: exclusive scan
@@ -1273,11 +1278,9 @@ void free_all(pirrt_graph *G) {
     if (G->pre_done) cudaEventDestroy(G->pre_done);
     if (G->pre_free) cudaEventDestroy(G->pre_free);
     if (G->hargs) cudaFreeHost(G->hargs);
-    void *bufs[] = {G->dargs, G->pexport, G->rows, G->ralloc, G->touched, G->roff, G->adj[0], G->adj[1], G->g, G->g32, G->p, G->pc,
-                    G->deg, G->tile_sums, G->stamp, G->list[0], G->list[1], G->switched,
-                    G->dg, G->anc[0], G->anc[1], G->acc[0], G->acc[1], G->wx[0], G->wx[1], G->done, G->wl[0],
-                    G->wl[1], G->wstamp, G->swstamp, G->cand, G->aq, G->aring, G->ctr, G->stage, G->h,
-                    G->items[0], G->items[1], G->rec[0], G->rec[1], G->walk_words};
+    void *bufs[] = {G->dargs, G->rows, G->adj[0], G->adj[1], G->g, G->g32, G->p, G->pc, G->deg,
+                    G->tile_sums, G->stamp, G->list[0], G->list[1], G->dg, G->wstamp, G->swstamp,
+                    G->cand, G->aq, G->aring, G->ctr, G->stage, G->h, G->scratch, G->walk_words};
     for (void *q : bufs)
         if (q) cudaFree(q);
     if (G->ctr_host) cudaFreeHost(G->ctr_host);
@@ -1445,9 +1448,6 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
         }                                                                               \
     } while (0)
     ALLOC(G->rows, sizeof(RowExt) * nv);
-    ALLOC(G->ralloc, sizeof(int32_t) * (nv + 1));
-    ALLOC(G->touched, sizeof(int32_t) * nv);
-    ALLOC(G->roff, sizeof(int64_t) * (nv + 1));
     // A pool holds every row with room to grow plus the space rows moved out
     // of; a repack (1.25 x length + 2 per row) always fits.  The second pool
     // is allocated by the first repack.  +16 entries: a staged row copy is
@@ -1463,17 +1463,7 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     ALLOC(G->stamp, sizeof(unsigned) * nv);
     ALLOC(G->list[0], sizeof(int32_t) * nv);
     ALLOC(G->list[1], sizeof(int32_t) * nv);
-    ALLOC(G->switched, sizeof(int32_t) * nv);
     ALLOC(G->dg, sizeof(int32_t) * nv);
-    ALLOC(G->anc[0], sizeof(int32_t) * nv);
-    ALLOC(G->anc[1], sizeof(int32_t) * nv);
-    ALLOC(G->acc[0], sizeof(double) * nv);
-    ALLOC(G->acc[1], sizeof(double) * nv);
-    ALLOC(G->wx[0], sizeof(longlong2) * nv);
-    ALLOC(G->wx[1], sizeof(longlong2) * nv);
-    ALLOC(G->done, sizeof(int32_t) * nv);
-    ALLOC(G->wl[0], sizeof(int32_t) * nv);
-    ALLOC(G->wl[1], sizeof(int32_t) * nv);
     ALLOC(G->wstamp, sizeof(unsigned) * nv);
     ALLOC(G->swstamp, sizeof(unsigned) * nv);
     ALLOC(G->cand, sizeof(unsigned long long) * nv);
@@ -1481,13 +1471,41 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     ALLOC(G->aring, sizeof(AsyncItem) * nv);
     ALLOC(G->ctr, sizeof(DevCounters));
     ALLOC(G->dargs, kArgBytes);
-    ALLOC(G->pexport, sizeof(int32_t) * nv);
     ALLOC(G->walk_words, kWalkBarBytes);
     if (cudaMemset(G->walk_words, 0, kWalkBarBytes) != cudaSuccess) return bail(PIRRT_ERR_CUDA);
-    for (int k = 0; k < 2; ++k) {
-        ALLOC(G->items[k], sizeof(WaveItem) * nv);
-        ALLOC(G->rec[k], sizeof(JumpRec) * nv);
-    }
+    // The arrays of each use lie one after another from the block's start; with no
+    // block yet, the bytes they take.
+    const auto carve = [&](int use) {
+        size_t at = 0;
+        const auto take = [&](auto &ptr, size_t count) {
+            using T = std::remove_reference_t<decltype(*ptr)>;
+            if (G->scratch) ptr = reinterpret_cast<T *>(static_cast<char *>(G->scratch) + at);
+            at += (sizeof(T) * count + 255) & ~size_t(255);
+        };
+        if (use == 0) {
+            take(G->roff, nv + 1);
+            take(G->ralloc, nv + 1);
+            take(G->touched, nv);
+            take(G->pexport, nv);
+        } else if (use == 1) {
+            for (int k = 0; k < 2; ++k) {
+                take(G->items[k], nv);
+                take(G->rec[k], nv);
+            }
+        } else {
+            take(G->switched, nv);
+            take(G->done, nv);
+            for (int k = 0; k < 2; ++k) {
+                take(G->acc[k], nv);
+                take(G->wx[k], nv);
+                take(G->anc[k], nv);
+                take(G->wl[k], nv);
+            }
+        }
+        return at;
+    };
+    ALLOC(G->scratch, std::max({carve(0), carve(1), carve(2)}));
+    for (int use = 0; use < 3; ++use) carve(use);
 #undef ALLOC
     if (cudaMallocHost((void **)&G->hargs, kArgBytes) != cudaSuccess) return bail(PIRRT_ERR_OOM);
     if (cudaStreamCreateWithFlags(&G->copy, cudaStreamNonBlocking) != cudaSuccess ||
