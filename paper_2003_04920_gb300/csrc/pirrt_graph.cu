@@ -103,6 +103,8 @@ struct pirrt_graph {
     int async_dirty = 0;                  // an exploit failed: reset the walk state first
     int32_t *pexport = nullptr;           // parents as reported (root marker -> -1)
     int deep_hint = 0;                    // AUTO: recent exploits met waves past the cap
+    int64_t fresh = 0;                    // AUTO: entries inserted since the last exploit
+    int whole = 0;                        // ... or the whole policy is new to it
     float *h = nullptr;                   // goal-directed Replan: heuristic h(v), cap_n entries
     int32_t goal = -1;                    // x_goal; -1 = goal-free
     int stale = 0;        // an exploit pruned subtrees: some g below them are not up to date
@@ -837,6 +839,7 @@ pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const i
     }
     G->n = n_after;
     G->m = m_after;
+    G->fresh += 2 * n_edges;
     return PIRRT_OK;
 }
 
@@ -849,6 +852,15 @@ pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const i
 // this size), so that only deeper vertices get reassociated sums.
 constexpr int64_t kJumpVertices = 1000000, kJumpVerticesF64 = 20000;
 constexpr int kTopRounds = 8;
+// Above kJumpAlways vertices a block of less than 1/kFewShare of the edges changes too
+// little for that: AUTO takes the wave there, as on larger graphs, until one is deep
+// (2-D), and tries again every kFewProbe exploits.  An exploit by jumping / by waves
+// in us, blocks of 100 vertices in 6-D: 300,000 vertices 216 / 131, 950,000 457 / 144;
+// blocks of 1,000 there 605 / 281, of 1/80 702 / 549.  Up to 2*10^5 vertices the two
+// differ by 60 us at most in 6-D (179 / 119), and in 2-D jumping wins by more than that
+// (399 / 838).
+constexpr int64_t kJumpAlways = 200000, kFewShare = 200;
+constexpr int kFewProbe = 64;
 
 // The default exploit: the whole Replan loop as one cooperative launch
 // (replan_loop.cuh).  One host wait, no read-back copy: the kernel leaves its
@@ -1004,16 +1016,19 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
     const bool async = mode == PIRRT_EVAL_ASYNC;
     const unsigned max_levels = (mode == PIRRT_EVAL_WAVE || mode == PIRRT_EVAL_ASYNC) ? cap_any
                                 : (o.wave_levels > 0 ? (unsigned)o.wave_levels : auto_cap);
-    // AUTO: after an exploit whose waves ran past the cap, use pointer
-    // jumping; probe with a wave again every eighth exploit
-    bool jump = mode == PIRRT_EVAL_JUMP ||
-                (mode == PIRRT_EVAL_AUTO && G->deep_hint && (G->exploits % 8) != 0);
     const bool one_launch = G->profiling != 1 && o.host_loop == 0 && tile == 0 && !async &&
                             (gs == 0 || gs == (sizeof(CT) == 8 ? 8 : 4));
     // (its pointer jumping only: the other forms' costs more than their wave up to
     // twice, 17.0 against 9.9 ms on 150,000 vertices in 2-D with tile 2)
-    const bool small = one_launch && mode == PIRRT_EVAL_AUTO && G->goal < 0 &&
+    const bool jumps = one_launch && mode == PIRRT_EVAL_AUTO && G->goal < 0 &&
                        G->n <= (sizeof(CT) == 8 ? kJumpVerticesF64 : kJumpVertices);
+    const bool few = jumps && G->n > kJumpAlways && !G->whole && G->fresh * kFewShare < G->m;
+    const bool small = jumps && !few;
+    // AUTO: after an exploit whose waves ran past the cap, use pointer
+    // jumping; probe with a wave again every eighth exploit
+    bool jump = mode == PIRRT_EVAL_JUMP ||
+                (mode == PIRRT_EVAL_AUTO && G->deep_hint &&
+                 (G->exploits % (few ? kFewProbe : 8)) != 0);
     if (small) jump = true;
     G->exploits += 1;
     // one CTA walks levels of at most this many vertices (~34 CSR entries each
@@ -1224,6 +1239,7 @@ pirrt_status set_policy_impl(pirrt_graph *G, const int32_t *parent) {
     begin_exploit_kernel<<<1, 1, 0, G->stream>>>(G->ctr, 1u, 0ull);
     CKL();
     G->stale = 0;
+    G->whole = 1;
     return PIRRT_OK;
 }
 
@@ -1247,6 +1263,7 @@ pirrt_status reevaluate_impl(pirrt_graph *G) {
     CK(cudaMemcpyAsync(&G->ctr->dense, &one, sizeof(unsigned), cudaMemcpyHostToDevice, G->stream));
     CK(cudaStreamSynchronize(G->stream));
     G->stale = 0;
+    G->whole = 1;
     return PIRRT_OK;
 }
 
@@ -1632,6 +1649,8 @@ pirrt_status pirrt_graph_reset(pirrt_graph *G) {
     G->args_key = pirrt_graph::ArgsKey{};
     G->deep_hint = 0;
     G->exploits = 0;
+    G->fresh = 0;
+    G->whole = 0;
     G->stale = 0;
     G->goal_dirty = 0;
     G->recover = 0;
@@ -1795,6 +1814,7 @@ pirrt_status pirrt_graph_exploit(pirrt_graph *G, const pirrt_exploit_opts *opts,
     const pirrt_status rc = G->cfg.cost_dtype == PIRRT_COST_F32 ? exploit_impl<float>(G, opts, stats)
                                                                 : exploit_impl<double>(G, opts, stats);
     if (rc != PIRRT_OK) G->async_dirty = 1;
+    else G->fresh = G->whole = 0;
     return rc;
 }
 
@@ -2055,6 +2075,7 @@ pirrt_status load_impl(pirrt_graph *G, FILE *f, const CkptHeader &h) {
     G->n = n;
     G->m = m;
     G->pool_used = m;
+    G->whole = 1;
     return PIRRT_OK;
 }
 }  // extern "C++"
@@ -2261,7 +2282,8 @@ struct TrialRunner {
     pirrt_batch *B;
     pirrt_graph *G;
     StateSnapshot snap;
-    int deep0 = 0, expl0 = 0;
+    int deep0 = 0, expl0 = 0, whole0 = 0;
+    int64_t fresh0 = 0;
     unsigned wave_epoch_max = 0;
     int trials = 0;
 
@@ -2273,7 +2295,16 @@ struct TrialRunner {
         if ((rc = snapshot_io(G, snap, true))) return rc;
         deep0 = G->deep_hint;
         expl0 = G->exploits;
+        fresh0 = G->fresh;
+        whole0 = G->whole;
         return PIRRT_OK;
+    }
+
+    void host_state() {
+        G->deep_hint = deep0;
+        G->exploits = expl0;
+        G->fresh = fresh0;
+        G->whole = whole0;
     }
 
     // One exploit with `o` from the saved state; its time in *ms.
@@ -2286,8 +2317,7 @@ struct TrialRunner {
                                cudaMemcpyHostToDevice, G->stream));
         }
         ++trials;
-        G->deep_hint = deep0;
-        G->exploits = expl0;
+        host_state();
         pirrt_exploit_stats st{};
         rc = pirrt_graph_exploit(G, &o, &st);
         if (rc == PIRRT_OK) {
@@ -2308,8 +2338,7 @@ struct TrialRunner {
                 rc = PIRRT_ERR_CUDA;
         }
         cudaStreamSynchronize(G->stream);
-        G->deep_hint = deep0;
-        G->exploits = expl0;
+        host_state();
         if (snap.buf) cudaFree(snap.buf);
         snap.buf = nullptr;
         return rc;
