@@ -98,7 +98,8 @@ typedef struct {
     int32_t wave_tail;      /* top-down Evaluate: grid steps of at most this many vertices
                                are walked by one CTA, with no level limit and no grid barrier;
                                0 = tuned, < 0 = off */
-    int32_t wave_ctas;      /* top-down Evaluate: CTAs per SM (1 or 2); 0 = tuned */
+    int32_t wave_ctas;      /* the loop, or its top-down Evaluate: CTAs per SM (1 or 2); 0 =
+                               tuned (policies walked in shared memory always take 1) */
     int32_t wave_local;     /* top-down Evaluate: tree levels a CTA walks on its own, from the
                                children it lowered, before they join the next grid step;
                                0 = tuned, < 0 = none (one level per grid step) */

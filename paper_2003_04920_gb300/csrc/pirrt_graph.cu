@@ -139,7 +139,7 @@ struct pirrt_graph {
     JumpRec *rec[2] = {nullptr, nullptr};     // ... pointer-jumping records (also set_policy's)
     static_assert(sizeof(JumpRec) == sizeof(WalkRec), "one array serves both");
     LoopResult *loop_res = nullptr;           // ... what an exploit reports (pinned)
-    int loop_occ = 0;                         // ... CTAs per SM (<= 2)
+    int loop_occ = 0, loop_occ64 = 0;         // ... CTAs per SM (<= 2), FP32 and FP64 costs
     int eval_blocks = 0;
     int wave_blocks = 0;                  // grid of the wave for the current exploit
     int wave_occ = 0;                     // CTAs per SM the wave can keep resident (<= 2)
@@ -861,13 +861,44 @@ constexpr int kTopRounds = 8;
 // (399 / 838).
 constexpr int64_t kJumpAlways = 200000, kFewShare = 200;
 constexpr int kFewProbe = 64;
+// Two CTAs of 64 registers per SM, which spill but keep twice the loads in flight, where
+// an exploit goes over much of a large graph: pointer jumping above kTwoJump vertices,
+// waves above kTwoWave after a block of at least 1/kManyShare of the edges or a new
+// policy.  Exploit time with one over that with two, blocks of all / a half / an eighth
+// / a 64th of the vertices: jumping, 300,000 vertices in 6-D 1.02 0.93 1.00 0.96 (2-D
+// 1.10 1.05 1.05 1.04), 600,000 1.10 0.99 1.07 1.03 (1.21 1.14 1.13 1.12); waves,
+// 1,200,000 in 6-D 1.03 1.06 0.99 0.88, 4,000,000 1.18 1.11 1.07 0.94 (2-D, from
+// scratch with one CTA walking thin steps, 0.87).
+constexpr int64_t kTwoJump = 500000, kTwoWave = 1000000, kManyShare = 8;
+
+// Most CTAs per SM of the one-launch loop, and its shared memory (with one, also that of
+// the largest policy walked there).
+template <typename CT>
+cudaError_t loop_setup(int *occ) {
+    constexpr int64_t most = sizeof(CT) == 4 ? kWalkVertices : kWalkVerticesF64;
+    const int smem = (int)sizeof(LoopShared<CT>);
+    int one = 0, two = 0;
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(replan_loop_kernel<CT, 1>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  smem + 16 + (int)walk_bytes<CT>(most))) ||
+        (e = cudaFuncSetAttribute(replan_loop_kernel<CT, 2>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&one, replan_loop_kernel<CT, 1>,
+                                                           kLoopThreads, smem)) ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&two, replan_loop_kernel<CT, 2>,
+                                                           kLoopThreads, smem)))
+        return e;
+    *occ = two >= 2 ? 2 : one >= 1 ? 1 : 0;
+    return cudaSuccess;
+}
 
 // The default exploit: the whole Replan loop as one cooperative launch
 // (replan_loop.cuh).  One host wait, no read-back copy: the kernel leaves its
 // report in page-locked host memory.
 template <typename CT>
 pirrt_status exploit_loop(pirrt_graph *G, const pirrt_exploit_opts &o, bool jump, bool adaptive,
-                          int top_rounds, int64_t max_iters, unsigned dense_limit, unsigned max_levels,
+                          int ctas, int top_rounds, int64_t max_iters, unsigned dense_limit, unsigned max_levels,
                           pirrt_exploit_stats *st) {
     LoopArgs<CT> a{};
     a.rows = G->rows;
@@ -903,15 +934,15 @@ pirrt_status exploit_loop(pirrt_graph *G, const pirrt_exploit_opts &o, bool jump
     a.local_levels = o.wave_local < 0 ? 0u : (o.wave_local > 0 ? (unsigned)o.wave_local : 32u);
     a.local_max = o.wave_local_max > 0 ? (unsigned)o.wave_local_max : 32u;
     a.local_step = o.wave_local_step > 0 ? (unsigned)o.wave_local_step : 512u;
-    const int occ = o.wave_ctas > 0 ? std::min(o.wave_ctas, G->loop_occ) : G->loop_occ;
-    int blocks = G->num_sms * occ;
     // a policy that fits shared memory is walked there, with the CTAs that leaves
     // every one its share of the vertices (loop_walk)
     constexpr int per = sizeof(CT) == 4 ? kWalkPer : kWalkPerF64;
     constexpr int64_t most = sizeof(CT) == 4 ? kWalkVertices : kWalkVerticesF64;
     a.walk = G->n <= std::min<int64_t>(most, (int64_t)per * G->num_sms) ? 1 : 0;
     const int64_t share = a.walk ? per : 128;
-    blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(8, (G->n + share - 1) / share));
+    const int occ = a.walk ? 1 : std::min(ctas, sizeof(CT) == 4 ? G->loop_occ : G->loop_occ64);
+    const int blocks = (int)std::min<int64_t>((int64_t)G->num_sms * occ,
+                                              std::max<int64_t>(8, (G->n + share - 1) / share));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(kLoopThreads);
@@ -925,7 +956,7 @@ pirrt_status exploit_loop(pirrt_graph *G, const pirrt_exploit_opts &o, bool jump
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     CK(cudaEventRecord(G->ev0, G->stream));
-    CK(cudaLaunchKernelEx(&cfg, replan_loop_kernel<CT>, a));
+    CK(cudaLaunchKernelEx(&cfg, occ == 2 ? replan_loop_kernel<CT, 2> : replan_loop_kernel<CT, 1>, a));
     CK(cudaEventRecord(G->ev1, G->stream));
     CK(cudaStreamSynchronize(G->stream));
     G->prof.launches += 1;
@@ -1041,8 +1072,11 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
         o.wave_local < 0 ? 0u : (o.wave_local > 0 ? (unsigned)o.wave_local : 32u);
     const unsigned local_max = o.wave_local_max > 0 ? (unsigned)o.wave_local_max : 128u;
     const unsigned local_step = o.wave_local_step > 0 ? (unsigned)o.wave_local_step : 4096u;
+    const bool many = G->whole || G->fresh * kManyShare >= G->m;
+    const int loop_ctas = o.wave_ctas > 0 ? o.wave_ctas
+                          : (jump ? G->n > kTwoJump : G->n > kTwoWave && many) ? 2 : 1;
     if (one_launch)
-        return exploit_loop<CT>(G, o, jump, mode == PIRRT_EVAL_AUTO && !small,
+        return exploit_loop<CT>(G, o, jump, mode == PIRRT_EVAL_AUTO && !small, loop_ctas,
                                 small ? kTopRounds : 0, max_iters, dense_limit, max_levels, st);
     pirrt_status rc = insertion_ended(G);
     if (rc) return rc;
@@ -1571,23 +1605,9 @@ pirrt_status pirrt_graph_create(const pirrt_config *cfg, pirrt_graph **out) {
     if (wocc < 1) return bail(PIRRT_ERR_CUDA);
     G->wave_occ = std::min(wocc, 2);
     G->wave_blocks = G->num_sms * G->wave_occ;
-    int locc = 0, locc64 = 0;
-    if (cudaFuncSetAttribute(
-            replan_loop_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-            (int)(sizeof(LoopShared<float>) + 16 + walk_bytes<float>(kWalkVertices))) != cudaSuccess ||
-        cudaFuncSetAttribute(
-            replan_loop_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-            (int)(sizeof(LoopShared<double>) + 16 + walk_bytes<double>(kWalkVerticesF64))) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&locc, replan_loop_kernel<float>, kLoopThreads,
-                                                      sizeof(LoopShared<float>)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&locc64, replan_loop_kernel<double>,
-                                                      kLoopThreads, sizeof(LoopShared<double>)) !=
-            cudaSuccess)
+    if (loop_setup<float>(&G->loop_occ) != cudaSuccess ||
+        loop_setup<double>(&G->loop_occ64) != cudaSuccess || G->loop_occ < 1 || G->loop_occ64 < 1)
         return bail(PIRRT_ERR_CUDA);
-    locc = std::min(locc, locc64);
-    if (locc < 1) return bail(PIRRT_ERR_CUDA);
-    G->loop_occ = std::min(locc, 2);
     int iocc = 0, iocc64 = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&iocc, insert_kernel<float>, kInsertThreads,
                                                       0) != cudaSuccess ||
@@ -2423,7 +2443,7 @@ pirrt_status pirrt_batch_autotune_search(pirrt_batch *B, const pirrt_exploit_opt
                       cur.evaluate != PIRRT_EVAL_ASYNC && cur.host_loop == 0;
     if (cur.group == 0) cur.group = lanes;
     if (cur.dense_fraction == 0.0) cur.dense_fraction = 0.35;
-    if (cur.wave_ctas == 0) cur.wave_ctas = 2;
+    if (cur.wave_ctas == 0) cur.wave_ctas = loop && G->n <= kTwoJump ? 1 : 2;
     if (cur.wave_local == 0) cur.wave_local = 32;
     if (cur.wave_local_max == 0) cur.wave_local_max = loop ? 32 : 128;
     if (cur.wave_local_step == 0) cur.wave_local_step = loop ? 512 : 4096;

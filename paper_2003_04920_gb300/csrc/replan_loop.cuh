@@ -11,9 +11,10 @@
 //   * a grid barrier carries a count, so the size of the next list needs no
 //     further round trip (2,100 cycles with 16 CTAs, 2,350 with 152);
 //   * one CTA of 512 threads per SM, 128 registers a thread: two CTAs of 64
-//     registers spilled in every phase (2-D queries of 10^4 vertices 18.5 against
-//     16.5 ms; at 4*10^6 vertices the two are even), and small graphs get as many
-//     CTAs as they have work for;
+//     registers spill in every phase (2-D queries of 10^4 vertices 18.5 against
+//     16.5 ms), so they are taken only where an exploit goes over much of a large
+//     graph and the loads in flight count; small graphs get as many CTAs as they
+//     have work for;
 //   * a switched vertex enters the Evaluate with the value Improve computed for
 //     it and its row extent, so Evaluate's first level starts at the row;
 //   * rows are classified first and their atomics issued by class; few vertices
@@ -1300,8 +1301,8 @@ __device__ __forceinline__ void loop_mark(const LoopArgs<CT> &a, LoopCounters *i
     flush_marks<CT>(sh, next, &ic->n_next);
 }
 
-template <typename CT>
-__global__ void __launch_bounds__(kLoopThreads, 1)
+template <typename CT, int OCC>  // CTAs per SM
+__global__ void __launch_bounds__(kLoopThreads, OCC)
 replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
     LoopShared<CT> &sh = loop_shared<CT>();
     DevCounters *c = a.ctr;
