@@ -127,8 +127,10 @@ typedef struct {
  *            cost-to-come (Sec. V policy improvement).  Same sums, bit for bit.
  *   AUTO  -- without a goal, JUMP on graphs of up to 10^6 vertices (FP64 costs:
  *            2 * 10^4, with the sums of the top 96 tree levels taken root to
- *            leaf); else WAVE, handing over to JUMP when a wave exceeds its
- *            level cap. */
+ *            leaf) and, with FP32 costs, on larger ones after a new policy (but
+ *            above 2 * 10^5 vertices after a block of less than 1/200 of the
+ *            edges as on larger graphs); else WAVE, handing over to JUMP when a
+ *            wave exceeds its level cap. */
 enum { PIRRT_EVAL_AUTO = 0, PIRRT_EVAL_WAVE = 1, PIRRT_EVAL_JUMP = 2, PIRRT_EVAL_ASYNC = 3 };
 
 /* Filled by pirrt_graph_exploit. */

@@ -847,6 +847,11 @@ pirrt_status insert_impl(pirrt_graph *G, int64_t n_new, int64_t n_edges, const i
 // grows with the graph (20 us an iteration at 2*10^5 vertices, 50 at 10^6) where
 // a wave's is the depth of the change (40 to 130 us on the 2-D and 6-D roadmaps).
 // With a goal the wave prunes and pointer jumping does not.
+// After a policy handed in most vertices switch, and a wave then goes over most of
+// the graph level by level: with FP32 costs AUTO jumps at any size (from breadth-first
+// trees, waves / jumping: 3*10^6 vertices in 6-D 15.0 / 9.7 ms, 1.5*10^6 in 2-D with
+// the level cap 62 / 16, random graphs of 3*10^6 with rows of 8 and 32 entries 3.5 /
+// 2.8 and 7.3 / 4.4).
 // FP64 costs, whose sums round, first take kTopRounds rounds that add from the
 // root down like the wave (96 tree levels, the depth of 2-D roadmaps of about
 // this size), so that only deeper vertices get reassociated sums.
@@ -1052,7 +1057,8 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
     // (its pointer jumping only: the other forms' costs more than their wave up to
     // twice, 17.0 against 9.9 ms on 150,000 vertices in 2-D with tile 2)
     const bool jumps = one_launch && mode == PIRRT_EVAL_AUTO && G->goal < 0 &&
-                       G->n <= (sizeof(CT) == 8 ? kJumpVerticesF64 : kJumpVertices);
+                       (sizeof(CT) == 8 ? G->n <= kJumpVerticesF64
+                                        : G->n <= kJumpVertices || G->whole != 0);
     const bool few = jumps && G->n > kJumpAlways && !G->whole && G->fresh * kFewShare < G->m;
     const bool small = jumps && !few;
     // AUTO: after an exploit whose waves ran past the cap, use pointer
