@@ -1249,6 +1249,8 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
     return PIRRT_OK;
 }
 
+constexpr int64_t kTwoPolicy = 500000;  // two CTAs per SM above (set_policy.cuh)
+
 template <typename CT>
 pirrt_status set_policy_impl(pirrt_graph *G, const int32_t *parent) {
     PolicyArgs<CT> a{};
@@ -1267,10 +1269,12 @@ pirrt_status set_policy_impl(pirrt_graph *G, const int32_t *parent) {
     a.ctr = G->ctr;
     a.host = G->sig;
     a.seq = ++G->sig_seq;
-    const int blocks = grid_for(8 * G->n, kWalkThreads, std::min(G->num_sms, kWalkMaxBlocks));
+    const int ctas = G->n > kTwoPolicy ? 2 : 1;
+    const int blocks = grid_for(8 * G->n, kWalkThreads, std::min(ctas * G->num_sms, kWalkMaxBlocks));
+    const void *kernel = ctas == 2 ? (const void *)set_policy_kernel<CT, 2>
+                                   : (const void *)set_policy_kernel<CT, 1>;
     void *args[] = {&a};
-    CK(cudaLaunchCooperativeKernel((const void *)set_policy_kernel<CT>, dim3(blocks),
-                                   dim3(kWalkThreads), args, 0, G->stream));
+    CK(cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kWalkThreads), args, 0, G->stream));
     if (const pirrt_status rc = wait_host(G, &G->sig->seq, a.seq)) return rc;
     if (G->sig->status & kStatusBadInput)
         return fail(G, PIRRT_ERR_BAD_INPUT,

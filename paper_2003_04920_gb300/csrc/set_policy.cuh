@@ -9,7 +9,11 @@
 // word.
 // What bounds it is the row reads for large graphs, the barriers and the host's
 // part of the call for small ones.  2,000 vertices with FP64 costs: a call 102 us
-// before, 31 now.
+// before, 31 now.  Above 500,000 vertices two CTAs of 64 registers per SM, which spill
+// in the evaluation but keep more row reads in flight: with one / with two, rows of
+// 32 entries, FP32: 30,000 vertices 45 / 56 us, 300,000 152 / 124, 10^6 434 / 294, 3 10^6
+// 1214 / 781 (as separate launches 114, 181, 350, 818); rows of 8: 300,000 86 / 98,
+// 10^6 297 / 227.
 #pragma once
 
 #include "evaluate_walk.cuh"
@@ -35,8 +39,8 @@ struct PolicyArgs {
     unsigned seq;
 };
 
-template <typename CT>
-__global__ void __launch_bounds__(kWalkThreads, 1)
+template <typename CT, int OCC>  // CTAs per SM
+__global__ void __launch_bounds__(kWalkThreads, OCC)
 set_policy_kernel(const __grid_constant__ PolicyArgs<CT> a) {
     constexpr int L = 8;  // lanes per row
     const int lane = threadIdx.x & 31, gl = lane & (L - 1);
