@@ -261,15 +261,16 @@ constexpr int kQWarps = kT / 32;
 using Key = unsigned long long;
 constexpr Key kNoKey = ~0ull;
 
-// Ascending bitonic sort of 256 keys, element 32 r + lane in x[r] of a lane.
-__device__ __forceinline__ void sort256(Key (&x)[8], int lane) {
+// Ascending bitonic sort of 32 R keys, element 32 r + lane in x[r] of a lane.
+template <int R>
+__device__ __forceinline__ void sort_keys(Key (&x)[R], int lane) {
 #pragma unroll
-    for (int size = 2; size <= kBuf; size <<= 1) {
+    for (int size = 2; size <= 32 * R; size <<= 1) {
 #pragma unroll
         for (int dist = size >> 1; dist > 0; dist >>= 1) {
             if (dist >= 32) {
 #pragma unroll
-                for (int r = 0; r < 8; ++r) {
+                for (int r = 0; r < R; ++r) {
                     const int o = r ^ (dist >> 5);
                     if (o > r) {
                         const bool up = ((r * 32) & size) == 0;
@@ -280,7 +281,7 @@ __device__ __forceinline__ void sort256(Key (&x)[8], int lane) {
                 }
             } else {
 #pragma unroll
-                for (int r = 0; r < 8; ++r) {
+                for (int r = 0; r < R; ++r) {
                     const Key o = __shfl_xor_sync(0xffffffffu, x[r], dist);
                     const bool up = ((r * 32 + lane) & size) == 0;
                     const bool first = (lane & dist) == 0;
@@ -292,22 +293,35 @@ __device__ __forceinline__ void sort256(Key (&x)[8], int lane) {
     }
 }
 
-// Keep the k smallest of the buffer's cnt keys, sorted; limit becomes the k-th
-// key once there are k.
-__device__ __forceinline__ void keep_k(Key *buf, int &cnt, int k, Key &limit, int lane) {
-    __syncwarp();
-    Key x[8];
+// The first cnt <= 32 R keys of the buffer sorted.
+template <int R>
+__device__ __forceinline__ void sort_buffer(Key *buf, int cnt, int lane) {
+    Key x[R];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) x[r] = r * 32 + lane < cnt ? buf[r * 32 + lane] : kNoKey;
-    sort256(x, lane);
+    for (int r = 0; r < R; ++r) x[r] = r * 32 + lane < cnt ? buf[r * 32 + lane] : kNoKey;
+    sort_keys<R>(x, lane);
     __syncwarp();
 #pragma unroll
-    for (int r = 0; r < 8; ++r) buf[r * 32 + lane] = x[r];
+    for (int r = 0; r < R; ++r) buf[r * 32 + lane] = x[r];
+}
+
+// Keep the k smallest of the buffer's cnt keys, sorted (the first `kept` are what the
+// last call kept); limit becomes the k-th key once there are k.  The sort is as long as
+// the keys are many: 256 each time had made 20 neighbours of 10^6 points in the plane
+// 5.3 ms, as against the 3.3 of a thread per query with its sorted list.
+__device__ __forceinline__ void keep_k(Key *buf, int &cnt, int &kept, int k, Key &limit, int lane) {
+    if (cnt == kept) return;
+    __syncwarp();
+    if (cnt <= 32) sort_buffer<1>(buf, cnt, lane);
+    else if (cnt <= 64) sort_buffer<2>(buf, cnt, lane);
+    else if (cnt <= 128) sort_buffer<4>(buf, cnt, lane);
+    else sort_buffer<8>(buf, cnt, lane);
     __syncwarp();
     if (cnt >= k) {
         cnt = k;
         limit = buf[k - 1];
     }
+    kept = cnt;
 }
 
 // The k smallest (d2, id) among the grid's points with id < id_limit, other
@@ -328,7 +342,7 @@ __device__ int knn_search(const Grid &g, int k, const float (&q)[DIM], int qid, 
         slo[d] = 0;
         shi[d] = -1;
     }
-    int cnt = 0;
+    int cnt = 0, kept = 0;
     Key limit = kNoKey;
     bool scanned = false;
     for (int r = 1;; ++r) {
@@ -409,14 +423,14 @@ __device__ int knn_search(const Grid &g, int k, const float (&q)[DIM], int qid, 
                         if (m == 0u) continue;
                         if (in) buf[cnt + __popc(m & ((1u << lane) - 1u))] = key;
                         cnt += __popc(m);
-                        if (cnt > kBuf - 32) keep_k(buf, cnt, k, limit, lane);
+                        if (cnt > kBuf - 32) keep_k(buf, cnt, kept, k, limit, lane);
                     }
                 }
                 p0 = p2;
                 p1 = p3;
             }
         }
-        keep_k(buf, cnt, k, limit, lane);
+        keep_k(buf, cnt, kept, k, limit, lane);
 #pragma unroll
         for (int d = 0; d < DIM; ++d) {
             slo[d] = blo[d];
