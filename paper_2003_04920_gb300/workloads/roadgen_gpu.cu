@@ -442,15 +442,18 @@ __device__ int knn_search(const Grid &g, int k, const float (&q)[DIM], int qid, 
 }
 
 // One warp per point, in cell order (neighbouring warps scan the same cells): the
-// k nearest among all points.
+// k nearest among all points.  With `list`, of its *n_list points only.
 template <int DIM>
 __global__ void __launch_bounds__(kT)
 knn_kernel(long long n, Grid g, int k, const float *__restrict__ spts, const int *__restrict__ sid,
-           const long long *__restrict__ start, int *__restrict__ knn) {
+           const long long *__restrict__ start, int *__restrict__ knn, const int *__restrict__ list,
+           const int *__restrict__ n_list) {
     __shared__ Key s_buf[kQWarps][kBuf];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (long long s = (long long)blockIdx.x * kQWarps + warp; s < n;
-         s += (long long)gridDim.x * kQWarps) {
+    if (list) n = *n_list;
+    for (long long t = (long long)blockIdx.x * kQWarps + warp; t < n;
+         t += (long long)gridDim.x * kQWarps) {
+        const long long s = list ? list[t] : t;
         float q[DIM];
 #pragma unroll
         for (int d = 0; d < DIM; ++d) q[d] = spts[s * DIM + d];
@@ -459,6 +462,132 @@ knn_kernel(long long n, Grid g, int k, const float *__restrict__ spts, const int
         for (int a = lane; a < k; a += 32)
             knn[(long long)qid * k + a] = a < cnt ? (int)(unsigned)(s_buf[warp][a] & 0xffffffffull) : -1;
         __syncwarp();
+    }
+}
+
+// The same for few neighbours of many points: one thread per point with its list in
+// local memory, so that nothing is sorted and 32 queries share a warp.  Taken for up
+// to 24 neighbours in up to 4 dimensions, from 5,000 points per neighbour on (10,000 in
+// 4-D; six neighbours at least): us of the whole call, warp / thread, 10 neighbours of 10^5
+// points in 1, 2, 3, 4 dimensions 414 / 280, 678 / 309, 967 / 401, 1401 / 620; of 10^6 2272 /
+// 511, 4612 / 766, 7334 / 1299; 20 of 10^6 2268 / 1054, 4690 / 1757, 8062 / 3023.  Below
+// that there are too few threads (20 of 10^4: 253 / 273 in 1-D, 369 / 669 in 4-D), and
+// with more neighbours or dimensions lists and boxes are too long for a thread (24 of 10^5:
+// 677 / 583 in 2-D, 1422 / 1735 in 4-D; 10 of 10^5 in 8-D 12.2 / 19.7 ms).  A point whose
+// boxes hold far more points than a uniform spread gives goes to `late`, for a warp.
+constexpr int kThreadK = 24, kThreadDim = 4;
+bool by_thread(int dim, long long n, int k) {
+    return dim <= kThreadDim && k <= kThreadK &&
+           n >= (long long)(dim < 4 ? 5000 : 10000) * std::max(k, 6);
+}
+template <int DIM>
+__global__ void __launch_bounds__(kT)
+knn_thread_kernel(long long n, Grid g, int k, const float *__restrict__ spts,
+                  const int *__restrict__ sid, const long long *__restrict__ start,
+                  int *__restrict__ knn, int *__restrict__ late, int *__restrict__ n_late) {
+    const long long most = 128ll * k + 512;  // points looked at (uniform: up to 40 k)
+    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n;
+         s += (long long)gridDim.x * blockDim.x) {
+        long long seen = 0;
+        float q[DIM];
+        int qc[DIM], slo[DIM], shi[DIM];
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+            q[d] = spts[s * DIM + d];
+            qc[d] = cell_coord(g, q[d]);
+            slo[d] = 0;
+            shi[d] = -1;
+        }
+        const int qid = sid[s];
+        Key list[kThreadK];
+        int cnt = 0;
+        Key limit = kNoKey;  // the k-th key once there are k
+        bool scanned = false;
+        for (int r = 1;; ++r) {
+            // boxes of cells as in knn_search
+            int blo[DIM], bhi[DIM], c[DIM];
+            const float kth = __uint_as_float((unsigned)(limit >> 32));
+            const float w = sqrtf(kth) * 1.0001f + 1e-6f;
+            bool same = scanned, whole = true;
+#pragma unroll
+            for (int d = 0; d < DIM; ++d) {
+                if (cnt < k) {
+                    blo[d] = max(0, qc[d] - r);
+                    bhi[d] = min(g.G - 1, qc[d] + r);
+                } else {
+                    blo[d] = cell_coord(g, q[d] - w);
+                    bhi[d] = cell_coord(g, q[d] + w);
+                }
+                if (scanned) {
+                    blo[d] = min(blo[d], slo[d]);
+                    bhi[d] = max(bhi[d], shi[d]);
+                    same = same && blo[d] == slo[d] && bhi[d] == shi[d];
+                }
+                whole = whole && blo[d] == 0 && bhi[d] == g.G - 1;
+                c[d] = blo[d];
+            }
+            if (same && (cnt == k || whole)) break;
+            // every cell row of the box, less what the box before held
+            for (;;) {
+                long long id = 0, mul = g.G;
+                bool inside_old = scanned;
+                float box = 0.f;
+#pragma unroll
+                for (int d = 1; d < DIM; ++d) {
+                    id += (long long)c[d] * mul;
+                    mul *= g.G;
+                    inside_old = inside_old && c[d] >= slo[d] && c[d] <= shi[d];
+                    const float a0 = (float)(g.lo + c[d] * g.cw), a1 = (float)(g.lo + (c[d] + 1) * g.cw);
+                    const float e = q[d] < a0 ? a0 - q[d] : (q[d] > a1 ? q[d] - a1 : 0.f);
+                    box += e * e;
+                }
+                const float bound = __uint_as_float((unsigned)(limit >> 32)) * 1.0001f + 1e-6f;
+                if (cnt < k || !(box > bound)) {
+                    for (int part = 0; part < 2; ++part) {
+                        const int f = part == 0 ? blo[0] : inside_old ? shi[0] + 1 : bhi[0] + 1;
+                        const int l = part == 0 && inside_old ? slo[0] - 1 : bhi[0];
+                        if (f > l) continue;
+                        const long long p0 = start[id + f], p1 = start[id + l + 1];
+                        seen += p1 - p0;
+                        if (seen > most) break;
+                        for (long long p = p0; p < p1; ++p) {
+                            const int pid = sid[p];
+                            const Key key = ((Key)__float_as_uint(d2_of<DIM>(q, spts + p * DIM)) << 32) |
+                                            (unsigned)pid;
+                            if (pid == qid || key >= limit) continue;
+                            int at = cnt < k ? cnt++ : k - 1;
+                            for (; at > 0 && list[at - 1] > key; --at) list[at] = list[at - 1];
+                            list[at] = key;
+                            if (cnt == k) limit = list[k - 1];
+                        }
+                    }
+                }
+                if (seen > most) break;
+                int d = 1;
+#pragma unroll
+                for (; d < DIM; ++d) {
+                    if (c[d] < bhi[d]) {
+                        ++c[d];
+                        break;
+                    }
+                    c[d] = blo[d];
+                }
+                if (d == DIM) break;
+            }
+            if (seen > most) break;
+#pragma unroll
+            for (int d = 0; d < DIM; ++d) {
+                slo[d] = blo[d];
+                shi[d] = bhi[d];
+            }
+            scanned = true;
+        }
+        if (seen > most) {
+            late[atomicAdd(n_late, 1)] = (int)s;
+            continue;
+        }
+        for (int a = 0; a < k; ++a)
+            knn[(long long)qid * k + a] = a < cnt ? (int)(unsigned)(list[a] & 0xffffffffull) : -1;
     }
 }
 
@@ -872,7 +1001,11 @@ extern "C" int rgg_knn(int32_t dim, double lo, double hi, int64_t n, const doubl
     const size_t o_cell = m.add<long long>(n), o_start = m.add<long long>(cells + 1),
                  o_tiles = m.add<long long>((cells + 1) / kTile + 2), o_cnt = m.add<int>(cells + 1),
                  o_sid = m.add<int>(n), o_spts = m.add<float>((size_t)n * dim);
+    const bool threads = by_thread(dim, n, k);
+    const size_t o_late = m.add<int>(threads ? n + 1 : 1);
     if (!m.alloc()) return 2;
+    int *n_late = m.at<int>(o_late), *late = n_late + 1;
+    if (threads) RG_CK(cudaMemsetAsync(n_late, 0, sizeof(int), st));
     long long *cell_of = m.at<long long>(o_cell), *start = m.at<long long>(o_start),
               *tiles = m.at<long long>(o_tiles);
     int *cnt = m.at<int>(o_cnt), *sid = m.at<int>(o_sid);
@@ -885,8 +1018,14 @@ extern "C" int rgg_knn(int32_t dim, double lo, double hi, int64_t n, const doubl
     cell_scatter<<<grid_of(n), kT, 0, st>>>(n, dim, points, cell_of, start, cnt, spts, sid);
     RG_CKL();
     with_dim(dim, [&](auto D) {
-        knn_kernel<decltype(D)::value><<<grid_of(n * 32), kT, 0, st>>>(n, g, k, spts, sid, start,
-                                                                       knn);
+        constexpr int kDim = decltype(D)::value;
+        if constexpr (kDim <= kThreadDim) {
+            if (threads)
+                knn_thread_kernel<kDim><<<grid_of(n), kT, 0, st>>>(n, g, k, spts, sid, start, knn,
+                                                                   late, n_late);
+        }
+        knn_kernel<kDim><<<threads ? 152 * 4 : grid_of(n * 32), kT, 0, st>>>(
+            n, g, k, spts, sid, start, knn, threads ? late : nullptr, n_late);
     });
     RG_CKL();
     RG_CK(cudaStreamSynchronize(st));
