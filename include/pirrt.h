@@ -130,7 +130,8 @@ typedef struct {
  *            leaf) and, with FP32 costs, on larger ones after a new policy (but
  *            above 2 * 10^5 vertices after a block of less than 1/200 of the
  *            edges as on larger graphs); else WAVE, handing over to JUMP when a
- *            wave exceeds its level cap. */
+ *            wave exceeds its level cap, and JUMP in its place after iterations
+ *            that switch more than 1/8 of the vertices (FP32 costs, no goal). */
 enum { PIRRT_EVAL_AUTO = 0, PIRRT_EVAL_WAVE = 1, PIRRT_EVAL_JUMP = 2, PIRRT_EVAL_ASYNC = 3 };
 
 /* Filled by pirrt_graph_exploit. */

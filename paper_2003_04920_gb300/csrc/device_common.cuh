@@ -124,6 +124,7 @@ struct LoopCounters {
 struct LoopState {  // CTA 0's totals of one exploit, read by the CTA that reports
     unsigned long long switches;
     unsigned iter, converged, wave_levels, dense_sweeps, jump_rounds, jump_evals;
+    unsigned deep;  // waves that were finished by pointer jumping
 };
 
 // Device counters of one graph.  The host copies the block back once per

@@ -866,6 +866,14 @@ constexpr int kTopRounds = 8;
 // (399 / 838).
 constexpr int64_t kJumpAlways = 200000, kFewShare = 200;
 constexpr int kFewProbe = 64;
+// Between waves AUTO jumps after an iteration that switched more than 1/kMassShare of the
+// vertices (FP32 costs, no goal): a wave then goes over much of the graph in steps of
+// dependent random loads.  Exploit in ms, waves only / switches above a quarter, an
+// eighth, a 16th, a 64th: 4*10^6 vertices in 6-D, block of a half 29.6 / 14.8 14.5 14.5
+// 14.6, an eighth 9.9 / 9.9 7.3 7.2 7.3; 2*10^6 in 2-D, a half 56 / 33 29 26 22; random
+// graphs of 4*10^6 with rows of 32 entries, all 11.4 / 7.9 8.1 8.2 8.1, a quarter 1.21 /
+// 1.20 1.07 1.07 1.19, an eighth 0.59 / 0.59 0.60 0.65 0.79.
+constexpr int64_t kMassShare = 8;
 // Two CTAs of 64 registers per SM, which spill but keep twice the loads in flight, where
 // an exploit goes over much of a large graph: pointer jumping above kTwoJump vertices,
 // waves above kTwoWave after a block of at least 1/kManyShare of the edges or a new
@@ -903,7 +911,7 @@ cudaError_t loop_setup(int *occ) {
 // report in page-locked host memory.
 template <typename CT>
 pirrt_status exploit_loop(pirrt_graph *G, const pirrt_exploit_opts &o, bool jump, bool adaptive,
-                          int ctas, int top_rounds, int64_t max_iters, unsigned dense_limit, unsigned max_levels,
+                          bool mixed, int ctas, int top_rounds, int64_t max_iters, unsigned dense_limit, unsigned max_levels,
                           pirrt_exploit_stats *st) {
     LoopArgs<CT> a{};
     a.rows = G->rows;
@@ -930,6 +938,7 @@ pirrt_status exploit_loop(pirrt_graph *G, const pirrt_exploit_opts &o, bool jump
     a.list_cap = G->cap_n;
     a.root = G->cfg.root;
     a.jump = jump ? 1 : 0;
+    a.jump_above = mixed ? (unsigned)(G->n / kMassShare) : 0xffffffffu;
     a.top_rounds = top_rounds;
     a.hops = G->n <= 50000 ? 7 : (G->n <= 1000000 ? 3 : 2);
     a.max_iters = (unsigned)std::min<int64_t>(max_iters, 0xffffffffll);
@@ -970,7 +979,7 @@ pirrt_status exploit_loop(pirrt_graph *G, const pirrt_exploit_opts &o, bool jump
     CK(cudaEventElapsedTime(&ms, G->ev0, G->ev1));
     G->ctr_host->wave_epoch = r.wave_epoch;
     if (adaptive) {
-        const bool saw_deep = r.jump_evals > 0;
+        const bool saw_deep = jump ? r.jump_evals > 0 : r.deep > 0;
         if (saw_deep || !jump || (G->exploits % 8) == 1) G->deep_hint = saw_deep ? 1 : 0;
     }
     pirrt_exploit_stats s{};
@@ -1079,10 +1088,11 @@ pirrt_status exploit_impl(pirrt_graph *G, const pirrt_exploit_opts *opts, pirrt_
     const unsigned local_max = o.wave_local_max > 0 ? (unsigned)o.wave_local_max : 128u;
     const unsigned local_step = o.wave_local_step > 0 ? (unsigned)o.wave_local_step : 4096u;
     const bool many = G->whole || G->fresh * kManyShare >= G->m;
+    const bool mixed = sizeof(CT) == 4 && mode == PIRRT_EVAL_AUTO && G->goal < 0;
     const int loop_ctas = o.wave_ctas > 0 ? o.wave_ctas
                           : (jump ? G->n > kTwoJump : G->n > kTwoWave && many) ? 2 : 1;
     if (one_launch)
-        return exploit_loop<CT>(G, o, jump, mode == PIRRT_EVAL_AUTO && !small, loop_ctas,
+        return exploit_loop<CT>(G, o, jump, mode == PIRRT_EVAL_AUTO && !small, mixed, loop_ctas,
                                 small ? kTopRounds : 0, max_iters, dense_limit, max_levels, st);
     pirrt_status rc = insertion_ended(G);
     if (rc) return rc;

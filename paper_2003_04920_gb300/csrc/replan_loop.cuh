@@ -58,7 +58,7 @@ struct __align__(16) JumpRec {
 struct LoopResult {
     unsigned long long relax, improved, evaluated, offers, switches;
     unsigned iter, converged, status, wave_epoch;
-    unsigned wave_levels, dense_sweeps, jump_rounds, jump_evals;
+    unsigned wave_levels, dense_sweeps, jump_rounds, jump_evals, deep;
 };
 
 template <typename CT>
@@ -84,6 +84,7 @@ struct LoopArgs {
     int64_t list_cap;
     int32_t root;
     int32_t jump;         // every Evaluate by pointer jumping
+    unsigned jump_above;  // ... or those after more switches than this
     int32_t hops;         // links followed per pointer-jumping round
     int32_t top_rounds;   // FP64 costs: rounds summed from the root down before it
     int32_t walk;         // the policy fits shared memory: each vertex walks up to the root
@@ -1325,7 +1326,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
     unsigned la = c->la & 1u, epoch = c->epoch, tag = c->wave_epoch, par = c->loop_par & 1u;
     unsigned n_active = c->n_active;
     bool dense = c->dense != 0u, stale = c->g32_stale != 0u;
-    unsigned iter = 0, levels_sum = 0, dense_sum = 0, rounds_sum = 0, jump_sum = 0;
+    unsigned iter = 0, levels_sum = 0, dense_sum = 0, rounds_sum = 0, jump_sum = 0, deep_sum = 0;
     unsigned long long switches = 0;  // thread 0
     bool converged = false, ok = true;
     bool walk = a.walk != 0;  // ... until a policy is too deep for it
@@ -1392,9 +1393,9 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
         bool next_dense = false;
         unsigned levels = 0;
         int32_t *next = la ? a.list[0] : a.list[1];
-        if (tid == 0 && (n_sw == 0u || a.jump != 0)) trace_step(c, sh.tr, 0);
+        bool jump = a.jump != 0 || n_sw > a.jump_above;
+        if (tid == 0 && (n_sw == 0u || jump)) trace_step(c, sh.tr, 0);
         if (n_sw != 0u) {
-            bool jump = a.jump != 0;
             if (!jump) {
                 // ---- Evaluate, top-down in grid steps
                 int64_t count = (int64_t)n_sw;
@@ -1417,7 +1418,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
                     }
                     __syncthreads();
                     const bool tail = count <= (int64_t)a.tail_max;
-                    const bool walk = !stop && (tail || count <= (int64_t)a.local_step);
+                    const bool alone = !stop && (tail || count <= (int64_t)a.local_step);
                     const int64_t per = tail ? count : (count + gridDim.x - 1) / gridDim.x;
                     const int64_t lo = (int64_t)blockIdx.x * per < count
                                            ? (int64_t)blockIdx.x * per : count;
@@ -1428,7 +1429,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
                     unsigned made = 0;
                     if (lo < hi)
                         made = loop_step<CT>(a, ic, a.items[(t & 1u) ^ 1u], t == 0u, lo, hi,
-                                             !walk ? 0u : tail ? 0xffffffffu : a.local_levels,
+                                             !alone ? 0u : tail ? 0xffffffffu : a.local_levels,
                                              tail ? kStage : a.local_max);
                     ok = loop_sync<CT>(c, sh, made);
                     lost = stop;
@@ -1443,6 +1444,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
                 next_count = sh.v_next;
                 jump = (sh.v_flags & kLoopIncomplete) != 0u;
                 stale = true;
+                if (jump) ++deep_sum;
                 if (jump && next_dense) next_count = 0u;
             }
             if (jump) {
@@ -1509,6 +1511,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
             c->loop_state.dense_sweeps = dense_sum;
             c->loop_state.jump_rounds = rounds_sum;
             c->loop_state.jump_evals = jump_sum;
+            c->loop_state.deep = deep_sum;
             c->la = la;
             c->epoch = epoch;
             c->wave_epoch = tag;
@@ -1541,6 +1544,7 @@ replan_loop_kernel(const __grid_constant__ LoopArgs<CT> a) {
             r.dense_sweeps = __ldcg(&c->loop_state.dense_sweeps);
             r.jump_rounds = __ldcg(&c->loop_state.jump_rounds);
             r.jump_evals = __ldcg(&c->loop_state.jump_evals);
+            r.deep = __ldcg(&c->loop_state.deep);
             *a.res = r;
         }
     }
