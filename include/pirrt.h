@@ -25,7 +25,8 @@
  *     every buffer it passes; the library reads inputs before the call
  *     returns and never retains caller pointers, except
  *     pirrt_graph_prefetch_batch, whose copies read the host buffers after
- *     it returns (its comment gives how long they must stay).
+ *     it returns, and pirrt_graph_insert_batch, whose kernel may still be
+ *     reading device buffers then (their comments give how long they must stay).
  *   - All device work is ordered on the stream given at create time
  *     (NULL = legacy default stream).  Calls that return results to the
  *     host (exploit, get_*) return when that stream's work has been done.
@@ -90,9 +91,9 @@ typedef struct {
                                to pointer jumping; 0 = tuned */
     int32_t host_loop;      /* 1 = drive the Replan loop from the host, one counter read per
                                iteration; 0 = one launch for the whole loop (a cooperative
-                               kernel; with ASYNC, tile 1 .. 3 or other lane counts a CUDA
-                               graph whose WHILE node repeats Improve / Evaluate).  Profiling
-                               always uses the host loop. */
+                               kernel; with ASYNC, tile 1 .. 3 or a lane count other than the
+                               tuned one a CUDA graph whose WHILE node repeats Improve /
+                               Evaluate).  Profiling always uses the host loop. */
     double dense_fraction;  /* changed vertices, as a fraction of |V|, above which the next
                                Improve sweeps every vertex instead of a list; 0 = tuned */
     int32_t wave_tail;      /* top-down Evaluate: grid steps of at most this many vertices
@@ -190,8 +191,11 @@ pirrt_status pirrt_graph_reset(pirrt_graph *g);
  * Errors: PIRRT_ERR_CAPACITY, PIRRT_ERR_BAD_INPUT (ids outside
  * [0, n + n_new), src == dst, cost <= 0, NaN or Inf), PIRRT_ERR_OOM (the
  * second CSR pool could not be allocated); on error the graph is unchanged.
- * Synchronises the stream once to read the validation result and the pool
- * space the block needs (and once more when the pool is repacked). */
+ * Returns once the block has been validated and the pool room it takes is known
+ * (after a wait for the stream when the pool is repacked); the entries are written
+ * after that, on the graph's stream.  Host arrays have been copied by then; device
+ * arrays are read again and stay unchanged until that work has been done (work
+ * issued to the same stream afterwards may overwrite them). */
 pirrt_status pirrt_graph_insert_batch(pirrt_graph *g, int64_t n_new_vertices, int64_t n_edges,
                                       const int32_t *src, const int32_t *dst, const void *cost,
                                       int on_device);
@@ -341,8 +345,8 @@ typedef struct {
 
 /* Clear the profile and turn event timing on (enable = 1) or off (0).
  * enable = 2 keeps only the device-side wave trace (the level_*, share_*,
- * local_* and wave_* fields) and leaves every exploit a single CUDA-graph
- * launch, with no host loop and no events. */
+ * local_* and wave_* fields) and leaves every exploit a single launch, with
+ * no host loop and no events. */
 pirrt_status pirrt_graph_set_profiling(pirrt_graph *g, int enable);
 
 /* Copy the profile accumulated since the last pirrt_graph_set_profiling
@@ -430,7 +434,10 @@ pirrt_status pirrt_selftest_insert_timeout(pirrt_graph *g);
  * member b owns the vertex ids [base_b, base_b + max_vertices[b]) and its
  * own root.  Policy iteration on the union is policy iteration on every
  * member at once (no edge joins two members), so every member reaches
- * exactly the policy of its own Replan, bit for bit; the whole batch runs in
+ * the policy of its own Replan: bit for bit wherever the path sums are exact in
+ * FP64 (FP32 costs within some 29 binades) or both evaluate alike; otherwise g
+ * agrees within the rounding of the sums, since AUTO chooses WAVE or JUMP by the
+ * size of the union.  The whole batch runs in
  * one launch per exploit.  Inserts are staged per member and
  * merged into the device CSR in one pass at the next exploit (Sec. IV-A:
  * one CSR rebuild per Replan).

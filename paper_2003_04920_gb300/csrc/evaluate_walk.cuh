@@ -14,8 +14,8 @@
 // per SM (152 arrivals at a barrier instead of 1,216), fewer when the policy
 // is smaller than that.
 //
-// Measured, whole calls: 200,003 vertices 236 edges deep 123 -> 44 us, of
-// which the kernel 92 -> 27.  Links per round, at 3,000 / 200,003 / 262,144
+// Measured, whole calls: 200,003 vertices 236 edges deep 128 -> 44 us, of
+// which the kernel 92 -> 27.  Links per round (in one run), at 3,000 / 200,003 / 262,144
 // vertices (the last some 800 deep): two 39.8 / 48.2 / 56.6 us, four 38.3 /
 // 43.0 / 50.9, eight 42.1 / 49.4 / 62.1.  Three take 35.1 / 39.7 / 46.2, but
 // need two additions per factor of three in depth: with four links added in

@@ -11,7 +11,7 @@
 // is written to one page of static host memory, pinned by the first call: the
 // call synchronises its stream and finds it there, without a copy.  One launch
 // instead of four and the outcome without a copy took 200,003 vertices from
-// 123 to 44 us a call.
+// 128 to 44 us a call.
 #include <cuda_runtime.h>
 
 #include <atomic>

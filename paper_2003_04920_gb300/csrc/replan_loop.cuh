@@ -21,11 +21,11 @@
 //     take a warp each, many 8 lanes each (4*10^6 vertices: 73 ms of waves a
 //     schedule against 87 with a warp each);
 //   * pointer jumping follows several links between two barriers.
-// Measured against one launch per iteration in a CUDA-graph WHILE node (same
-// GPU, whole schedules, insertion included): 2-D query of 10^4 vertices toward a
-// goal, 100 blocks, 51.5 -> 23.7 ms; 2-D, 2*10^5 vertices, 20 blocks, 48.6 ->
-// 25.2 ms; 6-D toward a goal, 10^6 vertices, 17.9 -> 11.6 ms; 6-D, 4*10^6
-// vertices, 80 blocks, 164 -> 133 ms.
+// Whole schedules with one launch per iteration in a CUDA-graph WHILE node and seven
+// per insertion, and now (insert.cuh included; same GPU): 2-D query of 10^4 vertices
+// toward a goal, 100 blocks, 45.8 -> 18.0 ms; 2-D, 2*10^5 vertices, 20 blocks, 50.4 ->
+// 24.4 ms; 6-D toward a goal, 10^6 vertices, 14.6 -> 8.0 ms; 6-D, 4*10^6 vertices, 80
+// blocks, 163 -> 126 ms.
 #pragma once
 
 #include "graph_kernels.cuh"
